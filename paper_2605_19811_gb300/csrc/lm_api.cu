@@ -201,6 +201,11 @@ MuonConsts muon_consts(const lm_config& c) {
 }
 
 // Device-memory arena: one cudaMalloc, sub-allocated with 256-byte alignment.
+// An allocation is laid out by two arenas: the tables (small, built on the
+// host and copied whole) and behind them the buffers (momentum, X, A, B, ...:
+// gigabytes that only start at zero, so the device clears them; copying them
+// from a zeroed host image cost 4.1 of the 4.4 ms of a bf16 msign of a
+// 1280 x 5120 matrix, and seconds in lm_create of the 720M-shaped set).
 // With guard bands on (LM_DEBUG=1 when the state is created), every part is
 // followed by kGuardBytes of a fixed pattern, checked by lm_get_status.
 constexpr size_t kGuardBytes = 256;
@@ -433,7 +438,7 @@ static void plan_groups(const std::vector<std::pair<int64_t, int64_t>>& shapes, 
   }
 }
 
-// Reserve workspace for the groups and the tile lists in the arena.
+// Reserve workspace for the groups (arena buf) and the tile lists (arena ar).
 struct NsLayout {
   std::vector<size_t> off_x0, off_x1, off_a, off_b, off_xf;
   std::vector<std::vector<NsTile>> tiles;   // per batch*3 + phase
@@ -501,18 +506,18 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, std::ve
 
 // tiles_mode: 0 or 1 one-block tiles, 2 two-block tiles wherever a row has
 // two blocks left (bf16 operands).
-static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Arena& ar, NsLayout& L,
+static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Arena& ar, Arena& buf, NsLayout& L,
                       std::vector<NsBatch>& batches, int pieces = 1, int tiles_mode = 0) {
   const size_t es = dtype_size(xdt) * (size_t)pieces;
   for (auto& g : groups) {
     const size_t xb = (size_t)g.count * g.s_pad * g.l_pad * es;
     const size_t ab = (size_t)g.count * g.s_pad * g.s_pad * es;
-    L.off_x0.push_back(ar.add(xb));
-    L.off_x1.push_back(ar.add(xb));
-    L.off_a.push_back(ar.add(ab));
-    L.off_b.push_back(ar.add(ab));
+    L.off_x0.push_back(buf.add(xb));
+    L.off_x1.push_back(buf.add(xb));
+    L.off_a.push_back(buf.add(ab));
+    L.off_b.push_back(buf.add(ab));
     // three-piece mode: fp32 X_0 / X_K
-    L.off_xf.push_back(pieces == 3 ? ar.add((size_t)g.count * g.s_pad * g.l_pad * sizeof(float)) : 0);
+    L.off_xf.push_back(pieces == 3 ? buf.add((size_t)g.count * g.s_pad * g.l_pad * sizeof(float)) : 0);
   }
   const int per = (xdt == LM_BF16) ? kMaxGroupsTc : kMaxGroupsSimt;
   int max_split = 0;
@@ -581,16 +586,17 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
   L.off_groups = ar.add(groups.size() * sizeof(NsGroup));
   L.off_norm = ar.add((size_t)std::max(nmat, 1) * sizeof(double));
   const size_t tile_floats = (xdt == LM_BF16) ? (size_t)kTcBM * kTcBN : (size_t)kSimtBM * kSimtBN;
-  L.off_split_ws = ar.add((size_t)max_split * tile_floats * sizeof(float));
+  L.off_split_ws = buf.add((size_t)max_split * tile_floats * sizeof(float));
 }
 
-static void bind_ns(NsEngine& E, char* base, const NsLayout& L, std::vector<char>& host_img) {
+// base: start of the tables (image host_img), bbase: start of the buffers.
+static void bind_ns(NsEngine& E, char* base, char* bbase, const NsLayout& L, std::vector<char>& host_img) {
   for (size_t gi = 0; gi < E.groups.size(); ++gi) {
-    E.groups[gi].X[0] = base + L.off_x0[gi];
-    E.groups[gi].X[1] = base + L.off_x1[gi];
-    E.groups[gi].A = base + L.off_a[gi];
-    E.groups[gi].B = base + L.off_b[gi];
-    E.groups[gi].Xf = E.pieces == 3 ? base + L.off_xf[gi] : nullptr;
+    E.groups[gi].X[0] = bbase + L.off_x0[gi];
+    E.groups[gi].X[1] = bbase + L.off_x1[gi];
+    E.groups[gi].A = bbase + L.off_a[gi];
+    E.groups[gi].B = bbase + L.off_b[gi];
+    E.groups[gi].Xf = E.pieces == 3 ? bbase + L.off_xf[gi] : nullptr;
   }
   for (size_t bi = 0; bi < E.batches.size(); ++bi)
     for (int ph = 0; ph < 3; ++ph) {
@@ -626,7 +632,7 @@ static void bind_ns(NsEngine& E, char* base, const NsLayout& L, std::vector<char
     E.batches[bi].split_targets = reinterpret_cast<NsSplitTarget*>(base + L.off_split_targets[bi]);
     if (!st.empty()) memcpy(host_img.data() + L.off_split_targets[bi], st.data(), st.size() * sizeof(NsSplitTarget));
   }
-  E.d_split_ws = reinterpret_cast<float*>(base + L.off_split_ws);
+  E.d_split_ws = reinterpret_cast<float*>(bbase + L.off_split_ws);
   E.d_groups = reinterpret_cast<NsGroup*>(base + L.off_groups);
   memcpy(host_img.data() + L.off_groups, E.groups.data(), E.groups.size() * sizeof(NsGroup));
   E.d_norm2 = reinterpret_cast<double*>(base + L.off_norm);
@@ -989,9 +995,9 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   plan_groups(mat_shapes, s->ns.xdt, s->ns.groups, members);
   s->nmat = (int)mat_param.size();
 
-  // arena layout
-  Arena ar;
-  ar.guard = s->debug;
+  // arena layout: tables (ar), then buffers (buf)
+  Arena ar, buf;
+  ar.guard = buf.guard = s->debug;
   s->mom_off.resize(n);
   size_t mom_elems_aligned = 0;
   for (int i = 0; i < n; ++i) {
@@ -999,7 +1005,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
     mom_elems_aligned = align_up(mom_elems_aligned + (size_t)numel(params[i]), 64);
     s->mom_elems += (size_t)numel(params[i]);
   }
-  const size_t off_mom = ar.add(mom_elems_aligned * sizeof(float));
+  const size_t off_mom = buf.add(mom_elems_aligned * sizeof(float));
   // AdamW second moments of the 1-D parameters
   s->adamw = cfg->vector_rule == LM_VECTOR_ADAMW;
   s->v_off.assign(n, -1);
@@ -1011,7 +1017,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
         v_aligned = align_up(v_aligned + (size_t)numel(params[i]), 64);
         s->v_elems += (size_t)numel(params[i]);
       }
-  const size_t off_v = ar.add(v_aligned * sizeof(float));
+  const size_t off_v = buf.add(v_aligned * sizeof(float));
   const size_t off_grads = ar.add((size_t)n * sizeof(void*));
   const size_t off_flags = ar.add(sizeof(unsigned));
 
@@ -1076,7 +1082,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
 
   // Muon tables
   NsLayout L;
-  layout_ns(s->ns.groups, s->ns.xdt, s->nmat, ar, L, s->ns.batches, s->ns.pieces, env_tiles_mode());
+  layout_ns(s->ns.groups, s->ns.xdt, s->nmat, ar, buf, L, s->ns.batches, s->ns.pieces, env_tiles_mode());
   s->ns.pdl = !env_is("LM_PDL", "0");
   s->ns.fold = !env_is("LM_NS_FOLD", "0");
   s->ns.wait_ns = env_wait_limit_ns();
@@ -1190,29 +1196,34 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
 
   size_t off_guard_list = 0;
   std::vector<size_t> guard_offs;
+  if (s->debug)
+    off_guard_list = ar.add((ar.guards.size() + buf.guards.size() + 1) * sizeof(size_t));
+  const size_t off_buf = align_up(ar.total, 256);   // the buffers follow the tables
+  const size_t total = off_buf + buf.total;
   if (s->debug) {
-    off_guard_list = ar.add(ar.guards.size() * sizeof(size_t) + sizeof(size_t));
     guard_offs = ar.guards;   // now including the list's own guard
+    for (size_t g : buf.guards) guard_offs.push_back(off_buf + g);
   }
   if (env_is("LM_FAULT", "oom")) {
     delete s;
     return fail(LM_ERR_OOM, "injected allocation failure (LM_FAULT=oom)");
   }
-  cudaError_t e = cudaMalloc(&s->base, ar.total);
+  cudaError_t e = cudaMalloc(&s->base, total);
   if (e != cudaSuccess) {
     delete s;
     return cuda_fail(e, "cudaMalloc(state)");
   }
-  s->bytes = ar.total;
+  s->bytes = total;
   std::vector<char> img(ar.total, 0);
   if (s->debug) {
-    for (size_t g : guard_offs) memset(img.data() + g, kGuardByte, kGuardBytes);
+    for (size_t g : ar.guards) memset(img.data() + g, kGuardByte, kGuardBytes);
     memcpy(img.data() + off_guard_list, guard_offs.data(), guard_offs.size() * sizeof(size_t));
     s->d_guard_offs = reinterpret_cast<size_t*>(s->base + off_guard_list);
     s->n_guards = (int)guard_offs.size();
   }
   char* base = s->base;
-  s->mom = reinterpret_cast<float*>(base + off_mom);
+  char* bbase = s->base + off_buf;
+  s->mom = reinterpret_cast<float*>(bbase + off_mom);
   s->d_grads = reinterpret_cast<const void**>(base + off_grads);
   s->d_flags = reinterpret_cast<unsigned*>(base + off_flags);
 
@@ -1235,7 +1246,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
                       reinterpret_cast<LionChunk*>(base + off_lc_vec[d]), (int)lc_vec[d].size()};
     s->lion_grid[d] = lion_grid_size((lm_dtype)d);
   }
-  s->vmom = reinterpret_cast<float*>(base + off_v);
+  s->vmom = reinterpret_cast<float*>(bbase + off_v);
   for (int d = 0; d < 2; ++d) {
     for (auto& t : at[d]) {
       t.m = s->mom + s->mom_off[t.pad];
@@ -1247,7 +1258,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
                   (int)ac[d].size()};
   }
 
-  bind_ns(s->ns, base, L, img);
+  bind_ns(s->ns, base, bbase, L, img);
   const bool f32x = s->ns.pieces == 3;   // X_0 and X_K in the fp32 buffer Xf
   const size_t es = f32x ? sizeof(float) : dtype_size(s->ns.xdt);
   for (size_t gi = 0; gi < s->ns.groups.size(); ++gi) {
@@ -1340,8 +1351,11 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   s->d_echunks[0] = reinterpret_cast<ElemChunk*>(base + off_echunks);
   s->d_echunks[1] = s->d_echunks[0] + s->n_echunks[0];
 
-  // Upload tables and zeros (momentum M_{-1} = 0, workspace padding = 0).
+  // Upload the tables; clear the buffers (momentum M_{-1} = 0, workspace padding = 0).
   e = cudaMemcpyAsync(base, img.data(), ar.total, cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess && buf.total > 0) e = cudaMemsetAsync(bbase, 0, buf.total, stream);
+  for (size_t k = 0; e == cudaSuccess && k < buf.guards.size(); ++k)
+    e = cudaMemsetAsync(bbase + buf.guards[k], kGuardByte, kGuardBytes, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     cudaFree(s->base);
@@ -1807,9 +1821,9 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   const lm_dtype xio = E.pieces == 3 ? LM_F32 : E.xdt;   // X_0 / X_K buffer dtype
   std::vector<std::vector<int>> members;
   plan_groups({{in->rows, in->cols}}, E.xdt, E.groups, members);
-  Arena ar;
+  Arena ar, buf;
   NsLayout L;
-  layout_ns(E.groups, E.xdt, 1, ar, L, E.batches, E.pieces, env_tiles_mode());
+  layout_ns(E.groups, E.xdt, 1, ar, buf, L, E.batches, E.pieces, env_tiles_mode());
   E.pdl = !env_is("LM_PDL", "0");
   E.fold = !env_is("LM_NS_FOLD", "0");
   E.wait_ns = env_wait_limit_ns();
@@ -1823,11 +1837,12 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   const size_t off_et = ar.add(et.size() * sizeof(ElemChunk));
   const size_t off_flags = ar.add(sizeof(unsigned));
 
+  const size_t off_buf = align_up(ar.total, 256);
   char* base = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), ar.total, stream);
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), off_buf + buf.total, stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(msign workspace)");
   std::vector<char> img(ar.total, 0);
-  bind_ns(E, base, L, img);
+  bind_ns(E, base, base + off_buf, L, img);
   const NsGroup& g = E.groups[0];
   d.w = in->data;
   d.m = nullptr;
@@ -1848,6 +1863,12 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   };
   e = cudaMemcpyAsync(base, img.data(), ar.total, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "msign table upload"));
+  // The buffer the norm kernel writes X_0 into must read as zero outside the
+  // matrix's true extent; every other buffer is written before it is read.
+  if (g.s != g.s_pad || g.l != g.l_pad) {
+    e = cudaMemsetAsync(d.x, 0, (size_t)g.s_pad * g.l_pad * dtype_size(xio), stream);
+    if (e != cudaSuccess) return cleanup(cuda_fail(e, "msign workspace clear"));
+  }
   if ((st = encode_maps(E)) != LM_OK) return cleanup(st);
   MuonConsts mk;
   memset(&mk, 0, sizeof(mk));
@@ -1862,11 +1883,14 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   if ((st = run_ns(E, steps, co.data(), dflags, stream)) != LM_OK) return cleanup(st);
   e = launch_finalize(xio, out->dtype, dm, de, (int)et.size(), mk, 1, dflags, stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "output kernel launch"));
-  // the call's status word: read back before the workspace goes
+  // The call's status word, read back before the workspace goes.  The
+  // workspace is freed after the synchronisation: the stream-ordered pool then
+  // still has it for a call that follows, and gives it back to the device at
+  // the program's next synchronisation.
   unsigned hflags = 0;
   e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, stream);
-  cudaFreeAsync(base, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  cudaFreeAsync(base, stream);
   if (e != cudaSuccess) return cuda_fail(e, "msign status read");
   if (hflags & LM_FLAG_TIMEOUT)
     return fail(LM_ERR_TIMEOUT, "a bounded device wait gave up; out was not written (LM_FLAG_TIMEOUT)");
