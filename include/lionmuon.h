@@ -85,7 +85,8 @@ typedef struct {
  *                       CTA pair (the default is one block); same results bit
  *                       for bit, slower on the GPT-style parameter sets
  *   LM_PDL=0            no programmatic dependent launch between the
- *                       Newton-Schulz launches (same results)
+ *                       Newton-Schulz launches of LM_NS_TILES=wide (same
+ *                       results; the default runs them as one launch)
  *   LM_NS_FOLD=0        bf16 Newton-Schulz keeps a X as a separate term of
  *                       X' = a X + B X; by default an iteration with |a| < 4
  *                       folds a into the diagonal of the stored B (results
@@ -381,7 +382,9 @@ lm_status lm_probe_bounded_wait(uint64_t limit_ns, uint32_t* device_flags,
                                 void* cuda_stream);
 
 /* Per-kernel-family timing, measured with CUDA events recorded on the
- * launching stream around every kernel launch of lm_step while enabled. */
+ * launching stream around every kernel launch of lm_step while enabled.  The
+ * tensor-core Newton-Schulz phases, otherwise one launch, then have a launch
+ * each (same results). */
 typedef enum {
   LM_KERNEL_LION = 0,          /* Lion step (all params, or vectors on Muon steps) */
   LM_KERNEL_MOMENTUM_NORM = 1, /* Muon: G_hat, ||G_hat||_F^2, M update, X0 */

@@ -277,10 +277,15 @@ struct NsBatch {
   int g0 = 0, ng = 0;
   NsTile* tiles[3] = {nullptr, nullptr, nullptr};
   int ntiles[3] = {0, 0, 0};
-  bool wide[3] = {false, false, false};            // tiles of two 256-column blocks: the wide-tile kernel
-  int* offsets[3] = {nullptr, nullptr, nullptr};   // per-pair tile ranges (tensor-core path)
-  int npairs[3] = {0, 0, 0};
+  bool wide = false;                               // tiles of two 256-column blocks: the wide-tile kernel
+  int* offsets[3] = {nullptr, nullptr, nullptr};   // per-pair tile ranges (tensor-core path), NULL: snake order
+  int npairs = 0;                                  // CTA pairs (tensor-core path)
+  int bn = kTcBN;                                  // columns of a tile (tensor-core path)
+  NsTile* compact[3] = {nullptr, nullptr, nullptr};   // masked steps: the selected matrices' tiles and their counts
+  int* counts = nullptr;
   NsSplitTarget* split_targets = nullptr;   // split Gram tiles of this batch
+  uint16_t* part_target = nullptr;          // target of each part
+  uint32_t* parts_done = nullptr;
   int nsplit = 0;
 };
 
@@ -389,11 +394,16 @@ struct NsEngine {
   int pieces = 1;                    // tensor cores: 3 = fp32 values as three bf16 planes
   std::vector<NsGroup> groups;       // host copies (device pointers inside)
   std::vector<TcGroupMaps> maps;     // tensor-core path
-  NsGroup* d_groups = nullptr;       // fp32 path reads groups from device memory
+  NsGroup* d_groups = nullptr;       // device copy (fp32 path, tile compaction)
   std::vector<NsBatch> batches;
+  // Cleared at the start of every step (clear_bytes from d_norm2): the norm
+  // accumulators, the chain kernel's three counters per matrix and its
+  // counters of the split Gram parts.
   double* d_norm2 = nullptr;
+  uint32_t* d_done = nullptr;
+  size_t clear_bytes = 0;
   float* d_split_ws = nullptr;       // fp32 partial sums of split Gram tiles
-  bool pdl = true;                   // programmatic dependent launch between NS launches
+  bool pdl = true;                   // programmatic dependent launch between wide-tile launches
   bool fold = true;                  // fold a into B's diagonal where |a| < 4 (bf16 operands)
   uint64_t wait_ns = kDefaultWaitNs; // limit of the kernels' bounded waits
 };
@@ -445,11 +455,16 @@ struct NsLayout {
   std::vector<size_t> off_tiles;
   std::vector<std::vector<int>> offsets;    // per batch*3 + phase (tensor-core path)
   std::vector<size_t> off_offsets;
+  std::vector<size_t> off_compact;          // per batch*3 + phase (masked steps)
+  std::vector<size_t> off_counts;           // per batch (masked steps)
   size_t off_groups = 0;
-  size_t off_norm = 0;
+  size_t off_clear = 0;
+  int nmat = 0, ntargets = 0;               // of the whole engine
   // split Gram tiles, per batch: (group, mat, tm, tn, first part, parts) of each target tile
   std::vector<std::vector<std::array<int, 6>>> split_targets;
   std::vector<size_t> off_split_targets;
+  std::vector<std::vector<uint16_t>> part_target;   // per batch
+  std::vector<size_t> off_part_target;
   size_t off_split_ws = 0;
 };
 
@@ -465,22 +480,50 @@ struct NsLayout {
 // most kcap: the three-piece fp32 mode bounds the length of each fp32
 // accumulation in TMEM that way (the parts are added in fp32 by the finish
 // kernel).
-static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, std::vector<NsTile>& t, int kslice,
-                             int workers, std::vector<std::array<int, 6>>& targets, int& nparts_total,
+// Decided per group (all matrices of a group split alike) from its upper
+// tile x tile blocks, whatever the columns of the tiles in t, so that every
+// tile width splits the same blocks into the same parts (and gives the same
+// sums).
+static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng, std::vector<NsTile>& t, int tile,
+                             int kslice, int workers, std::vector<std::array<int, 6>>& targets, int& nparts_total,
                              int kcap = 0) {
-  int64_t total = 0;
-  for (const NsTile& x : t) total += (int64_t)(groups[g0 + x.group].l_pad / kslice) * (x.nh == 2 ? 2 : 1);
+  std::vector<int64_t> blocks(ng), len(ng);
+  int64_t total = 0, longest = 0;
+  for (int g = 0; g < ng; ++g) {
+    const NsGroup& G = groups[g0 + g];
+    const int64_t r = (G.s_pad + tile - 1) / tile;
+    blocks[g] = (int64_t)G.count * r * (r + 1) / 2;
+    len[g] = G.l_pad / kslice;
+    total += blocks[g] * len[g];
+    longest = std::max(longest, len[g]);
+  }
   const int64_t avg = total / std::max(1, workers);
   int64_t part = std::max<int64_t>(8, avg / 2);
+  // Where the whole list comes to less than 32 slices a worker, a second
+  // round of parts costs as much as the first: the shortest parts of at least
+  // 8 slices that leave one block or part per worker.
+  if (kcap <= 0 && avg < 32) {
+    for (part = 8; part < longest; ++part) {
+      int64_t n = 0;
+      for (int g = 0; g < ng; ++g) n += (len[g] + part - 1) / part * blocks[g];
+      if (n <= workers) break;
+    }
+  }
+  const int64_t keep = avg < 32 ? std::max<int64_t>(2 * avg, part) : 2 * avg;   // tiles up to this length stay whole
   if (kcap > 0) part = std::min<int64_t>(part, kcap);
+  std::vector<char> whole(ng, 0);
+  int64_t planned = 0;   // part numbers are 16 bits (a block may be two tiles wide)
+  for (int g = 0; g < ng; ++g) {
+    const int64_t n = 2 * blocks[g] * std::min<int64_t>(64, (len[g] + part - 1) / part);
+    whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || planned + n > 65535;
+    if (!whole[g]) planned += n;
+  }
   std::vector<NsTile> out;
   nparts_total = 0;
   for (const NsTile& x0 : t) {
-    const int nk = groups[g0 + x0.group].l_pad / kslice;
+    const int64_t nk = len[x0.group];
     const int nh = x0.nh == 2 ? 2 : 1;
-    // decided per 256-column block, so that one- and two-block tiles split
-    // the same blocks into the same parts (and give the same sums)
-    if ((nk <= 2 * avg && (kcap <= 0 || nk <= kcap)) || nparts_total + 128 > 65535) {
+    if (whole[x0.group]) {
       out.push_back(x0);
       continue;
     }
@@ -493,8 +536,8 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, std::ve
       targets.push_back({x.group, x.mat, x.tm, x.tn, nparts_total, nparts});
       for (int k = 0; k < nparts; ++k) {
         NsTile y = x;
-        y.kb0 = (uint16_t)((int64_t)nk * k / nparts);
-        y.kb1 = (uint16_t)((int64_t)nk * (k + 1) / nparts);
+        y.kb0 = (uint16_t)(nk * k / nparts);
+        y.kb1 = (uint16_t)(nk * (k + 1) / nparts);
         y.slot = (uint16_t)(nparts_total + k + 1);
         out.push_back(y);
       }
@@ -504,10 +547,17 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, std::ve
   t.swap(out);
 }
 
+// Bytes of the block cleared at the start of a step: per matrix the norm
+// accumulator and three tile counters, per split target one counter.
+static size_t ns_clear_bytes(int nmat, int ntargets) {
+  return (size_t)nmat * (sizeof(double) + 3 * sizeof(uint32_t)) + (size_t)ntargets * sizeof(uint32_t);
+}
+
 // tiles_mode: 0 or 1 one-block tiles, 2 two-block tiles wherever a row has
 // two blocks left (bf16 operands).
 static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Arena& ar, Arena& buf, NsLayout& L,
-                      std::vector<NsBatch>& batches, int pieces = 1, int tiles_mode = 0) {
+                      std::vector<NsBatch>& batches, int pieces = 1, int tiles_mode = 0, bool masked = false,
+                      bool narrow_ok = true) {
   const size_t es = dtype_size(xdt) * (size_t)pieces;
   for (auto& g : groups) {
     const size_t xb = (size_t)g.count * g.s_pad * g.l_pad * es;
@@ -522,42 +572,65 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
   const int per = (xdt == LM_BF16) ? kMaxGroupsTc : kMaxGroupsSimt;
   int max_split = 0;
   const int bm = (xdt == LM_BF16) ? kTcBM : kSimtBM;
-  const int bn = (xdt == LM_BF16) ? kTcBN : kSimtBN;
   for (int g0 = 0; g0 < (int)groups.size(); g0 += per) {
     NsBatch b;
     b.g0 = g0;
     b.ng = std::min(per, (int)groups.size() - g0);
+    // Two-block tiles stage a quarter fewer bytes per FLOP, but they take
+    // both accumulators (the epilogue of one tile no longer overlaps the
+    // next tile's main loop), leave room for a 3- or 4-stage ring only and
+    // put twice as many matrices in flight in a launch (a larger L2 working
+    // set): measured slower on the GPT-style sets, so used only on request.
+    b.wide = xdt == LM_BF16 && pieces == 1 && tiles_mode == 2;
+    if (xdt == LM_BF16) {
+      int64_t apply_tiles = 0;   // of 256 x 256
+      for (int gi = g0; gi < g0 + b.ng; ++gi)
+        apply_tiles += (int64_t)groups[gi].count * ((groups[gi].s_pad + kTcBM - 1) / kTcBM) * (groups[gi].l_pad / kTcBN);
+      b.bn = b.wide || !narrow_ok ? kTcBN : tc_tile_cols((int)std::min<int64_t>(apply_tiles, 1 << 30), pieces);
+    }
+    const int bn = (xdt == LM_BF16) ? b.bn : kSimtBN;
+    std::vector<NsTile> lists[3];
+    std::vector<std::array<int, 6>> targets;
+    for (int ph = 0; ph < 3; ++ph) build_ns_tiles(groups, g0, b.ng, ph, bm, bn, lists[ph], b.wide);
+    int nparts = 0;
+    if (xdt == LM_BF16) {
+      // three-piece mode: no fp32 accumulation over more than kGramCapF32TC K blocks
+      split_gram_tiles(groups, g0, b.ng, lists[NS_GRAM], kTcBM, kTcBK, tc_max_pairs(), targets, nparts,
+                       pieces == 3 ? kGramCapF32TC : 0);
+    } else {
+      int dev = 0, sms = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      split_gram_tiles(groups, g0, b.ng, lists[NS_GRAM], kSimtBM, 16, 2 * std::max(sms, 1), targets, nparts);
+    }
+    b.nsplit = (int)targets.size();
+    max_split = std::max(max_split, nparts);
+    L.ntargets += b.nsplit;
+    std::vector<uint16_t> pt((size_t)nparts);
+    for (size_t k = 0; k < targets.size(); ++k)
+      for (int q = 0; q < targets[k][5]; ++q) pt[(size_t)targets[k][4] + q] = (uint16_t)k;
+    // tiles per matrix, from each group's first matrix
+    for (int gi = g0; gi < g0 + b.ng; ++gi) {
+      NsGroup& g = groups[gi];
+      auto mine = [&](const NsTile& x) { return x.group == gi - g0 && x.mat == 0; };
+      g.n_gram = (int)std::count_if(lists[NS_GRAM].begin(), lists[NS_GRAM].end(),
+                                    [&](const NsTile& x) { return mine(x) && x.slot == 0; });
+      g.n_split = (int)std::count_if(targets.begin(), targets.end(), [&](const std::array<int, 6>& x) {
+        return x[0] == gi - g0 && x[1] == 0;
+      });
+      g.n_poly = (int)std::count_if(lists[NS_POLY].begin(), lists[NS_POLY].end(), mine);
+      g.n_apply = (int)std::count_if(lists[NS_APPLY].begin(), lists[NS_APPLY].end(), mine);
+    }
+    L.off_split_targets.push_back(ar.add(targets.size() * sizeof(NsSplitTarget)));
+    L.split_targets.push_back(std::move(targets));
+    L.off_part_target.push_back(ar.add(pt.size() * sizeof(uint16_t)));
+    L.part_target.push_back(std::move(pt));
+    if (xdt == LM_BF16)
+      b.npairs = (int)std::min<size_t>((size_t)tc_max_pairs(),
+                                       std::max(lists[0].size(), std::max(lists[1].size(), lists[2].size())));
     for (int ph = 0; ph < 3; ++ph) {
-      std::vector<NsTile> t;
-      build_ns_tiles(groups, g0, b.ng, ph, bm, bn, t);
-      // Two-block tiles stage a quarter fewer bytes per FLOP, but they take
-      // both accumulators (the epilogue of one tile no longer overlaps the
-      // next tile's main loop), leave room for a 3- or 4-stage ring only and
-      // put twice as many matrices in flight in a launch (a larger L2 working
-      // set): measured slower on the GPT-style sets, so used only on request.
-      if (xdt == LM_BF16 && pieces == 1 && tiles_mode == 2) {
-        t.clear();
-        build_ns_tiles(groups, g0, b.ng, ph, bm, bn, t, true);
-        b.wide[ph] = true;
-      }
+      std::vector<NsTile>& t = lists[ph];
       std::vector<int> offs;
-      std::vector<std::array<int, 6>> targets;
-      if (ph == NS_GRAM) {
-        int nparts = 0;
-        if (xdt == LM_BF16) {
-          // three-piece mode: no fp32 accumulation over more than kGramCapF32TC K blocks
-          split_gram_tiles(groups, g0, t, kTcBK, tc_max_pairs(), targets, nparts, pieces == 3 ? kGramCapF32TC : 0);
-        } else {
-          int dev = 0, sms = 0;
-          cudaGetDevice(&dev);
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-          split_gram_tiles(groups, g0, t, 16, 2 * std::max(sms, 1), targets, nparts);
-        }
-        b.nsplit = (int)targets.size();
-        max_split = std::max(max_split, nparts);
-        L.off_split_targets.push_back(ar.add(targets.size() * sizeof(NsSplitTarget)));
-        L.split_targets.push_back(std::move(targets));
-      }
       if (xdt == LM_BF16 && !t.empty()) {
         // cost of a tile: its K blocks plus an allowance for the epilogue
         std::vector<std::pair<int, NsTile>> sorted;
@@ -570,21 +643,29 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
                          [](const std::pair<int, NsTile>& a, const std::pair<int, NsTile>& c) {
                            return a.first > c.first;
                          });
-        const int workers = std::min<int>(tc_max_pairs(), (int)t.size());
         t.clear();
-        balance_tiles(sorted, workers, t, offs);
-        b.npairs[ph] = workers;
+        if (masked && !b.wide) {
+          // the list is compacted to the selected matrices on the device and
+          // dealt out in snake order, longest first
+          for (auto& x : sorted) t.push_back(x.second);
+        } else {
+          balance_tiles(sorted, std::min<int>(b.npairs, (int)sorted.size()), t, offs);
+          offs.resize((size_t)b.npairs + 1, offs.back());
+        }
       }
       b.ntiles[ph] = (int)t.size();
+      L.off_compact.push_back(masked && xdt == LM_BF16 ? ar.add(t.size() * sizeof(NsTile)) : 0);
       L.off_tiles.push_back(ar.add(t.size() * sizeof(NsTile)));
       L.tiles.push_back(std::move(t));
       L.off_offsets.push_back(ar.add(offs.size() * sizeof(int)));
       L.offsets.push_back(std::move(offs));
     }
+    L.off_counts.push_back(masked ? ar.add(3 * sizeof(int)) : 0);
     batches.push_back(b);
   }
   L.off_groups = ar.add(groups.size() * sizeof(NsGroup));
-  L.off_norm = ar.add((size_t)std::max(nmat, 1) * sizeof(double));
+  L.nmat = nmat;
+  L.off_clear = ar.add(std::max<size_t>(ns_clear_bytes(nmat, L.ntargets), 1));
   const size_t tile_floats = (xdt == LM_BF16) ? (size_t)kTcBM * kTcBN : (size_t)kSimtBM * kSimtBN;
   L.off_split_ws = buf.add((size_t)max_split * tile_floats * sizeof(float));
 }
@@ -604,29 +685,42 @@ static void bind_ns(NsEngine& E, char* base, char* bbase, const NsLayout& L, std
       E.batches[bi].tiles[ph] = reinterpret_cast<NsTile*>(base + L.off_tiles[k]);
       if (!L.tiles[k].empty())
         memcpy(host_img.data() + L.off_tiles[k], L.tiles[k].data(), L.tiles[k].size() * sizeof(NsTile));
+      if (L.off_compact[k] != 0) E.batches[bi].compact[ph] = reinterpret_cast<NsTile*>(base + L.off_compact[k]);
       if (!L.offsets[k].empty()) {
         E.batches[bi].offsets[ph] = reinterpret_cast<int*>(base + L.off_offsets[k]);
         memcpy(host_img.data() + L.off_offsets[k], L.offsets[k].data(), L.offsets[k].size() * sizeof(int));
       }
     }
+  E.d_norm2 = reinterpret_cast<double*>(base + L.off_clear);
+  E.d_done = reinterpret_cast<uint32_t*>(E.d_norm2 + L.nmat);
+  E.clear_bytes = ns_clear_bytes(L.nmat, L.ntargets);
+  uint32_t* parts_done = E.d_done + 3 * (size_t)L.nmat;
   for (size_t bi = 0; bi < E.batches.size(); ++bi) {
     const auto& tg = L.split_targets[bi];
+    E.batches[bi].parts_done = parts_done;
+    parts_done += tg.size();
+    E.batches[bi].part_target = reinterpret_cast<uint16_t*>(base + L.off_part_target[bi]);
+    if (!L.part_target[bi].empty())
+      memcpy(host_img.data() + L.off_part_target[bi], L.part_target[bi].data(),
+             L.part_target[bi].size() * sizeof(uint16_t));
+    if (L.off_counts[bi] != 0) E.batches[bi].counts = reinterpret_cast<int*>(base + L.off_counts[bi]);
     std::vector<NsSplitTarget> st(tg.size());
     const bool tc = E.xdt == LM_BF16;
     const size_t es = tc ? 2 : 4;                 // A: bf16 (tensor cores) or fp32
-    const int tile = tc ? kTcBM : kSimtBM;
+    const int tile = tc ? kTcBM : kSimtBM, tile_n = tc ? E.batches[bi].bn : kSimtBN;
     for (size_t k = 0; k < tg.size(); ++k) {
       const NsGroup& g = E.groups[E.batches[bi].g0 + tg[k][0]];
       char* a = static_cast<char*>(g.A) + (size_t)tg[k][1] * g.s_pad * g.s_pad * es;
       const int tm = tg[k][2], tn = tg[k][3];
-      st[k].a_tile = a + ((size_t)tm * tile * g.s_pad + (size_t)tn * tile) * es;
-      st[k].a_mirror = a + ((size_t)tn * tile * g.s_pad + (size_t)tm * tile) * es;
+      st[k].a_tile = a + ((size_t)tm * tile * g.s_pad + (size_t)tn * tile_n) * es;
+      st[k].a_mirror = a + ((size_t)tn * tile_n * g.s_pad + (size_t)tm * tile) * es;
       st[k].ld = g.s_pad;
       st[k].nr = std::min(tile, g.s_pad - tm * tile);
-      st[k].nc = std::min(tile, g.s_pad - tn * tile);
+      st[k].nc = std::min(tile_n, g.s_pad - tn * tile_n);
       st[k].first = tg[k][4];
       st[k].nparts = tg[k][5];
       st[k].diag = tm == tn ? 1 : 0;
+      st[k].mat = g.first_mat + tg[k][1];
       st[k].plane = (tc && E.pieces == 3) ? (int64_t)g.count * g.s_pad * g.s_pad : 0;
     }
     E.batches[bi].split_targets = reinterpret_cast<NsSplitTarget*>(base + L.off_split_targets[bi]);
@@ -635,16 +729,16 @@ static void bind_ns(NsEngine& E, char* base, char* bbase, const NsLayout& L, std
   E.d_split_ws = reinterpret_cast<float*>(bbase + L.off_split_ws);
   E.d_groups = reinterpret_cast<NsGroup*>(base + L.off_groups);
   memcpy(host_img.data() + L.off_groups, E.groups.data(), E.groups.size() * sizeof(NsGroup));
-  E.d_norm2 = reinterpret_cast<double*>(base + L.off_norm);
 }
 
 static lm_status encode_maps(NsEngine& E) {
   if (E.xdt != LM_BF16) return LM_OK;
   E.maps.resize(E.groups.size());
-  for (size_t gi = 0; gi < E.groups.size(); ++gi) {
-    cudaError_t e = tc_encode_group_maps(E.groups[gi], &E.maps[gi], E.pieces);
-    if (e != cudaSuccess) return cuda_fail(e, "cuTensorMapEncodeTiled");
-  }
+  for (const NsBatch& b : E.batches)
+    for (int gi = b.g0; gi < b.g0 + b.ng; ++gi) {
+      cudaError_t e = tc_encode_group_maps(E.groups[gi], &E.maps[gi], E.pieces, b.bn, b.wide);
+      if (e != cudaSuccess) return cuda_fail(e, "cuTensorMapEncodeTiled");
+    }
   return LM_OK;
 }
 
@@ -673,15 +767,19 @@ struct Profiler {
   }
 };
 
+// Whether launches on st are timed: profiling is on and the stream is not
+// being captured into a graph (the events would be graph nodes, not
+// measurements).
+static bool profiling(Profiler* P, cudaStream_t st) {
+  if (P == nullptr || !P->on) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return !(st != nullptr && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone);
+}
+
 // Launch f() on st; with profiling on, bracket it by events of family fam.
 template <typename F>
 static cudaError_t timed_events(Profiler* P, int fam, cudaStream_t st, F&& f) {
-  if (P == nullptr || !P->on) return f();
-  // launches being captured into a graph are not timed (their events would
-  // be graph nodes, not measurements)
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (st != nullptr && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
-    return f();
+  if (!profiling(P, st)) return f();
   cudaEvent_t a = P->next(), b = P->next();
   if (a == nullptr || b == nullptr) return f();
   cudaEventRecord(a, st);
@@ -724,43 +822,82 @@ static lm_status run_ns(const NsEngine& E, int steps, const NsCoeffs* coeffs, un
     });
     if (e != cudaSuccess) return cuda_fail(e, "three-piece split launch");
   }
-  for (int it = 0; it < steps; ++it)
-    for (const NsBatch& b : E.batches)
+  for (const NsBatch& b : E.batches) {
+    if (steps == 0) break;
+    if (E.xdt == LM_BF16 && !b.wide) {
+      NsChain c;
+      c.ngroups = b.ng;
+      c.groups = E.groups.data() + b.g0;
+      c.maps = E.maps.data() + b.g0;
+      c.counts = nullptr;
+      for (int ph = 0; ph < 3; ++ph) {
+        c.tiles[ph] = active ? b.compact[ph] : b.tiles[ph];
+        c.offsets[ph] = b.offsets[ph];
+        c.ntiles[ph] = b.ntiles[ph];
+      }
+      if (active) {   // the selected matrices' tiles
+        c.counts = b.counts;
+        cudaError_t e = timed(P, LM_KERNEL_OTHER, st, [&]() {
+          return launch_ns_compact(b.tiles, b.compact, b.ntiles, b.counts, E.d_groups + b.g0, active, flags, st);
+        });
+        if (e != cudaSuccess) return cuda_fail(e, "tile compaction launch");
+      }
+      c.npairs = b.npairs;
+      c.targets = b.split_targets;
+      c.part_target = b.part_target;
+      c.ntargets = b.nsplit;
+      c.parts_done = b.parts_done;
+      c.split_ws = E.d_split_ws;
+      c.done = E.d_done;
+      c.norm2 = E.d_norm2;
+      c.steps = steps;
+      c.co = coeffs;
+      c.fold = E.fold;
+      c.pieces = E.pieces;
+      c.bn = b.bn;
+      c.final_f32 = true;
+      c.fuse = fuse;
+      c.active = active;
+      c.flags = flags;
+      c.wait_ns = E.wait_ns;
+      // one launch for the whole chain; with profiling on, one per phase, so
+      // that every phase has a time of its own
+      if (!profiling(P, st)) {
+        cudaError_t e = launch_ns_chain(c, 0, 3 * steps, st);
+        if (e != cudaSuccess) return cuda_fail(e, "Newton-Schulz launch");
+        continue;
+      }
+      for (int q = 0; q < 3 * steps; ++q) {
+        if (q % 3 == NS_POLY && ns_iter_form(coeffs[q / 3], E.pieces, E.fold).from_a) continue;
+        cudaError_t e = timed(P, LM_KERNEL_NS_GRAM + q % 3, st, [&]() { return launch_ns_chain(c, q, q + 1, st); });
+        if (e != cudaSuccess) return cuda_fail(e, "Newton-Schulz launch");
+      }
+      continue;
+    }
+    for (int it = 0; it < steps; ++it)
       for (int ph = 0; ph < 3; ++ph) {
         const NsCoeffs co = coeffs[it];
-        // an iteration without the A^2 term (c = 0, a cubic): B = b A is not
-        // formed; the tensor-core APPLY reads A and scales by b instead
-        const bool from_a = E.xdt == LM_BF16 && co.c == 0.f && !b.wide[NS_POLY] && !b.wide[NS_APPLY];
-        if (ph == NS_POLY && from_a) continue;
-        // an iteration whose |a| is below 4: POLY stores B' = a I + B and APPLY
-        // computes X' = B' X with no X tile in its epilogue (bf16 operands,
-        // one-block tiles).  On the constant quintic this also lowers the
-        // error against the fp64 iteration (bf16 msign: 6.2e-3 against 8.3e-3
-        // on 1280 x 5120, 6.5e-3 against 1.0e-2 on 768 x 50304); a larger a
-        // (the first minimax iterations, 8.47) would round the diagonal too
-        // coarsely.
-        const bool fold = E.fold && E.xdt == LM_BF16 && E.pieces == 1 && !from_a && std::fabs(co.a) < 4.f &&
-                          !b.wide[NS_POLY] && !b.wide[NS_APPLY];
-        const bool split = E.xdt == LM_BF16 && ph == NS_GRAM && b.nsplit > 0;
+        const bool split = ph == NS_GRAM && b.nsplit > 0;
         cudaError_t e = timed(P, LM_KERNEL_NS_GRAM + ph, st, [&]() {
-          if (E.xdt == LM_BF16) {
-            cudaError_t r = launch_ns_tc((NsPhase)ph, it, b.ng, E.groups.data() + b.g0, E.maps.data() + b.g0, b.tiles[ph],
-                               b.ntiles[ph], b.offsets[ph], b.npairs[ph], E.d_norm2, co, flags,
-                               it == steps - 1 ? fuse : nullptr, st, active, split ? E.d_split_ws : nullptr,
-                               E.pieces, it == steps - 1 ? 1 : 0, b.wide[ph], E.pdl, E.wait_ns,
-                               ph == NS_APPLY && from_a, ph != NS_GRAM && fold);
+          if (b.wide) {
+            cudaError_t r = launch_ns_wide_phase((NsPhase)ph, it, b.ng, E.groups.data() + b.g0, E.maps.data() + b.g0,
+                                                 b.tiles[ph], b.ntiles[ph], b.offsets[ph],
+                                                 std::min(b.npairs, b.ntiles[ph]), E.d_norm2, co, flags,
+                                                 it == steps - 1 ? fuse : nullptr, st, active,
+                                                 split ? E.d_split_ws : nullptr, E.pdl, E.wait_ns);
             if (r == cudaSuccess && split)
               r = launch_ns_split_finish(b.split_targets, b.nsplit, E.d_split_ws, flags, st);
             return r;
           }
           cudaError_t r = launch_ns_simt((NsPhase)ph, it, b.ng, E.d_groups + b.g0, b.tiles[ph], b.ntiles[ph],
                                          E.d_norm2, co, st, active, E.d_split_ws, flags);
-          if (r == cudaSuccess && ph == NS_GRAM && b.nsplit > 0)
+          if (r == cudaSuccess && split)
             r = launch_ns_split_finish_f32(b.split_targets, b.nsplit, E.d_split_ws, flags, st);
           return r;
         });
         if (e != cudaSuccess) return cuda_fail(e, "Newton-Schulz launch");
       }
+  }
   return LM_OK;
 }
 
@@ -851,7 +988,7 @@ struct lm_state {
   int nmat = 0;
   MatDesc* d_mats = nullptr;
   bool fuse_final = false;   // parameter write in the last APPLY epilogue
-  CUtensorMap* d_wmaps = nullptr;   // TMA maps of every matrix's W (two each) for that write
+  CUtensorMap* d_wmaps = nullptr;   // TMA map of every matrix's W for that write
   ElemChunk* d_echunks[2] = {nullptr, nullptr};   // chunks of bf16 / fp32 matrices
   int n_echunks[2] = {0, 0};
   NsEngine ns;
@@ -1080,16 +1217,20 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
     off_lc_ema[d] = ar.add(lc_ema[d].size() * sizeof(LionChunk));
   }
 
-  // Muon tables
-  NsLayout L;
-  layout_ns(s->ns.groups, s->ns.xdt, s->nmat, ar, buf, L, s->ns.batches, s->ns.pieces, env_tiles_mode());
-  s->ns.pdl = !env_is("LM_PDL", "0");
+  // Muon tables.  A parameter write whose iteration does not fold a runs on
+  // 256-column tiles only.
   s->ns.fold = !env_is("LM_NS_FOLD", "0");
+  const bool narrow_ok = s->ns_co.empty() || ns_iter_form(s->ns_co.back(), s->ns.pieces, s->ns.fold).fold ||
+                         s->ns.pieces == 3;
+  NsLayout L;
+  layout_ns(s->ns.groups, s->ns.xdt, s->nmat, ar, buf, L, s->ns.batches, s->ns.pieces, env_tiles_mode(),
+            cfg->schedule == LM_SCHEDULE_STABLE_RANK, narrow_ok);
+  s->ns.pdl = !env_is("LM_PDL", "0");
   s->ns.wait_ns = env_wait_limit_ns();
   const size_t off_mats = ar.add((size_t)std::max(s->nmat, 1) * sizeof(MatDesc));
   // TMA maps of W for the parameter write in the last APPLY (bf16 tensor-core path)
   const bool want_wmaps = s->ns.xdt == LM_BF16 && s->ns.pieces == 1 && s->nmat > 0;
-  const size_t off_wmaps = want_wmaps ? ar.add((size_t)s->nmat * 2 * sizeof(CUtensorMap)) : 0;
+  const size_t off_wmaps = want_wmaps ? ar.add((size_t)s->nmat * sizeof(CUtensorMap)) : 0;
   std::vector<MatDesc> mats(s->nmat);
   // matrices are numbered in group order
   std::vector<int> mat_order;   // mat id -> index into mat_param
@@ -1344,7 +1485,7 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   if (s->fuse_final) {
     CUtensorMap* hm = reinterpret_cast<CUtensorMap*>(img.data() + off_wmaps);
     for (int id = 0; id < s->nmat && s->fuse_final; ++id)
-      if (tc_encode_w_maps(mats[id].w, mats[id].rows, mats[id].cols, hm + 2 * id) != cudaSuccess)
+      if (tc_encode_w_map(mats[id].w, mats[id].rows, mats[id].cols, hm + id) != cudaSuccess)
         s->fuse_final = false;   // finalize_kernel writes the parameters instead
     s->d_wmaps = reinterpret_cast<CUtensorMap*>(base + off_wmaps);
   }
@@ -1543,7 +1684,7 @@ lm_status lm_step(lm_state* s, const lm_tensor* grads, int n, int64_t t, void* c
   if (mixed) mk.active = s->d_active;
   if (s->nmat > 0) {
     e = timed(P, LM_KERNEL_OTHER, stream, [&]() {
-      return cudaMemsetAsync(s->ns.d_norm2, 0, (size_t)s->nmat * sizeof(double), stream);
+      return cudaMemsetAsync(s->ns.d_norm2, 0, s->ns.clear_bytes, stream);
     });
     if (e != cudaSuccess) return cuda_fail(e, "norm reset");
     for (int dt = 0; dt < 2; ++dt) {

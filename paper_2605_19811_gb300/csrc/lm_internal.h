@@ -135,6 +135,9 @@ struct NsGroup {
   int32_t s_pad, l_pad;   // padded sizes of the workspace buffers
   int32_t first_mat;      // index of the group's first matrix in the norm array
   int32_t tall;           // 1: X kept as l x s (rows > cols), 0: as s x l
+  // Tensor-core path, per matrix: whole Gram tiles, Gram tiles split along K,
+  // polynomial tiles, apply tiles (what the chain kernel's counters reach)
+  int32_t n_gram, n_split, n_poly, n_apply;
   int32_t pad_;
   void* X[2];             // ping-pong X: count x (s_pad x l_pad, or l_pad x s_pad if tall)
   void* A;                // count x s_pad x s_pad
@@ -145,7 +148,7 @@ struct NsGroup {
   void* Xf;
 };
 // Tile work item: group, matrix-in-group, tile row, tile col.
-struct NsTile {
+struct alignas(16) NsTile {
   uint16_t group, mat, tm, tn;
   // Split-K (Gram phase only): K blocks [kb0, kb1) of the tile, kb1 == 0 for
   // all of them; slot != 0: the partial product is written in fp32 to
@@ -168,6 +171,7 @@ struct NsSplitTarget {
   int32_t nr, nc;         // rows / columns of the tile inside the padded matrix
   int32_t first, nparts;
   int32_t diag;
+  int32_t mat;            // matrix id
   int64_t plane;          // three-piece A: elements between its bf16 planes (0: one bf16 plane)
 };
 constexpr int kMaxGroupsTc = 8;   // groups per tensor-core launch
@@ -179,24 +183,31 @@ struct NsCoeffs {
 // Tensor-core path (bf16 operands, fp32 accumulation in TMEM): one
 // kTcBM x kTcBN output tile per CTA pair; s is padded to 128, l to kTcBN.
 constexpr int kTcBM = 256, kTcBN = 256, kTcBK = 64;
+// Columns of a bf16 tile for a batch whose APPLY phase has `apply_tiles` tiles
+// of 256 x 256: 128 where that is at most one per CTA pair, 256 beyond.
+// Such a batch is bound by the latency of a tile, not by operand bytes: half
+// the columns halve its MMAs and its epilogue.  Three-piece operands always take
+// 128: their two accumulators (main and cross products) then fit TMEM twice, and
+// the epilogue of one tile overlaps the MMAs of the next.
+int tc_tile_cols(int apply_tiles, int pieces);
 int tc_pad_s(int s);
 int tc_pad_l(int l);
-// Tensor maps for one group: K-major boxes (64 x 128), MN-major boxes
-// (64 x 64) and store boxes (64 x 32) on X0, X1, A, B.  A and B hold only
-// their 256 x 256 tiles on or above the diagonal.
+// Tensor maps for one group.  A and B hold only their 256 x 256 tiles on or
+// above the diagonal.
 struct TcGroupMaps {
-  CUtensorMap xk[2];    // K-major operand / aux loads: box 64 x 128
-  CUtensorMap a;
-  CUtensorMap b;
-  CUtensorMap xmn[2];   // MN-major operand loads: 4-D box (64, 64, 2), a 128-wide half
-  CUtensorMap amn;      // transposed reads of stored A / B tiles: the same 4-D box
-  CUtensorMap bmn;
-  CUtensorMap xst[2];   // result stores: box 64 x 32
-  CUtensorMap ast;
-  CUtensorMap bst;
+  // A-operand loads, aux loads and result stores: 64 x 128 boxes, K-major;
+  // MN-major: 4-D box (64, 64, 2), a 128-wide half (transposed reads)
+  CUtensorMap xk[2], a, b;
+  CUtensorMap xmn[2], amn, bmn;
+  // B-operand loads: a CTA's half of the tile's columns (bn / 2 rows, or bn /
+  // 128 atoms of 64)
+  CUtensorMap nxk[2], na, nb;
+  CUtensorMap nxmn[2], namn, nbmn;
+  CUtensorMap xst[2], ast, bst;   // wide kernel: result stores, box 64 x 32
 };
-// pieces: 1 (bf16 buffers) or 3 (three bf16 planes per buffer)
-cudaError_t tc_encode_group_maps(const NsGroup& g, TcGroupMaps* maps, int pieces = 1);
+// pieces: 1 (bf16 buffers) or 3 (three bf16 planes per buffer); bn: columns of
+// a tile (256 or 128); wide: also the store maps of the wide kernel
+cudaError_t tc_encode_group_maps(const NsGroup& g, TcGroupMaps* maps, int pieces, int bn, bool wide);
 int tc_max_pairs();   // CTA pairs that fit the device (one CTA per SM)
 // One bounded wait on a barrier that is never signalled (failure-detection probe).
 cudaError_t launch_bounded_wait_probe(uint64_t limit_ns, unsigned* flags, cudaStream_t st);
@@ -206,41 +217,85 @@ cudaError_t launch_bounded_wait_probe(uint64_t limit_ns, unsigned* flags, cudaSt
 struct FuseFinal {
   const MatDesc* mats;
   float eM, lam;
-  // Two TMA maps per matrix (same index as mats), in device memory: W as
-  // 64 x 128 load boxes and 64 x 32 store boxes (tc_encode_w_maps).  Used
-  // where a is folded into B' (the APPLY then has no X tile to read).
+  // One TMA map per matrix (same index as mats), in device memory: W in 64 x
+  // 128 boxes, loaded and stored (tc_encode_w_map).  Used where a is folded
+  // into B' (the APPLY then has no X tile to read).
   const CUtensorMap* wmaps;
 };
-// The two W maps of FuseFinal::wmaps for one bf16 parameter (cols % 8 = 0).
-cudaError_t tc_encode_w_maps(void* w, int64_t rows, int64_t cols, CUtensorMap* maps);
+// The W map of FuseFinal::wmaps for one bf16 parameter (cols % 8 = 0).
+cudaError_t tc_encode_w_map(void* w, int64_t rows, int64_t cols, CUtensorMap* map);
 // Limit of a bounded device wait unless the state sets another
 // (LM_WAIT_LIMIT_NS at lm_create): a wait that runs out gives up and raises
 // LM_FLAG_TIMEOUT; every later kernel then does nothing until the flag is cleared.
 constexpr uint64_t kDefaultWaitNs = 5000000000ull;   // 5 s
 uint64_t env_wait_limit_ns();   // LM_WAIT_LIMIT_NS if set to a positive integer, else kDefaultWaitNs
-// offsets: NULL (round robin over tiles) or npairs + 1 range starts;
-// fuse: NULL, or the parameter write of the last APPLY phase;
-// apply_from_a: an APPLY of an iteration whose c is 0, whose POLY launch was
-// left out (B = b A): it reads A and scales its product by b (one-block
-// tiles only).
-cudaError_t launch_ns_tc(NsPhase ph, int iter, int ngroups, const NsGroup* groups,
-                         const TcGroupMaps* maps, const NsTile* tiles, int ntiles,
-                         const int* offsets, int npairs, const double* norm2, NsCoeffs co,
-                         unsigned* flags, const FuseFinal* fuse, cudaStream_t st,
-                         const unsigned char* active = nullptr, float* split_ws = nullptr, int pieces = 1,
-                         int final_f32 = 0, bool wide = false, bool pdl = false,
-                         uint64_t wait_ns = kDefaultWaitNs, bool apply_from_a = false, bool fold_a = false);
-// split_ws: non-NULL only for a Gram launch whose tiles include split-K parts.
-// pieces = 3: fp32 operands as three bf16 pieces (no split tiles, no fused
-// parameter write); final_f32: this APPLY writes fp32 X to NsGroup::Xf.
-// wide: the tile list may hold two-block tiles (NsTile::nh = 2), run by the
-// wide-tile kernel (bf16 only); pdl: programmatic dependent launch (the
-// kernel may start while the previous kernel on the stream finishes).
-// Both kernels do nothing when LM_FLAG_TIMEOUT is already set in *flags.
+constexpr int kMaxNsSteps = 64;
+// How an iteration is run on the tensor cores.  from_a: c = 0 (a cubic), so
+// B = b A is not formed and APPLY reads A and scales its product by b.
+// fold: POLY stores B' = a I + B and APPLY computes X' = B' X with no X tile
+// in its epilogue, for bf16 operands where |a| is below 4.  On the constant
+// quintic this also lowers the error against the fp64 iteration (bf16 msign:
+// 6.2e-3 against 8.3e-3 on 1280 x 5120, 6.5e-3 against 1.0e-2 on 768 x
+// 50304); a larger a (the first minimax iterations, 8.47) would round the
+// diagonal too coarsely.
+struct NsIterForm {
+  bool from_a, fold;
+};
+inline NsIterForm ns_iter_form(const NsCoeffs& co, int pieces, bool fold) {
+  const bool from_a = co.c == 0.f;
+  return NsIterForm{from_a, fold && pieces == 1 && !from_a && co.a < 4.f && co.a > -4.f};
+}
+// One batch of the chain kernel: every phase of every iteration of up to
+// kMaxGroupsTc groups.
+struct NsChain {
+  int ngroups;
+  const NsGroup* groups;        // host
+  const TcGroupMaps* maps;      // host
+  const NsTile* tiles[3];
+  const int* offsets[3];        // npairs + 1 range starts per phase, or NULL: the list dealt out in snake order
+  int ntiles[3];
+  const int* counts;            // device tile counts per phase (without offsets), or NULL: ntiles
+  int npairs;                   // CTA pairs, at most tc_max_pairs()
+  const NsSplitTarget* targets; // split Gram tiles, their parts' targets and counters, and the fp32 parts
+  const uint16_t* part_target;
+  int ntargets;
+  uint32_t* parts_done;         // zero before the first launch of a step
+  float* split_ws;
+  uint32_t* done;               // 3 counters per matrix id, zero before the first launch of a step
+  const double* norm2;
+  int steps;
+  const NsCoeffs* co;           // host, one per iteration
+  bool fold;
+  int pieces;                   // 1: bf16 operands; 3: fp32 as three bf16 pieces
+  int bn;                       // columns of a tile: 256, or 128 (always with three pieces; not with a parameter
+                                // write whose iteration does not fold a)
+  bool final_f32;               // three pieces: the last APPLY writes fp32 X to NsGroup::Xf
+  const FuseFinal* fuse;        // NULL, or the parameter write of the last APPLY (one piece)
+  const unsigned char* active;  // NULL, or the mask the tile lists were compacted by
+  unsigned* flags;
+  uint64_t wait_ns;
+};
+// Phases [q0, q1) of the sequence 3 * iteration + phase.  Does nothing when
+// LM_FLAG_TIMEOUT is already set in *flags.
+cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st);
+// Compact the tile lists of a masked step (src, n per phase) to the tiles of
+// selected matrices, with their counts.
+cudaError_t launch_ns_compact(const NsTile* const* src, NsTile* const* dst, const int* n, int* counts,
+                              const NsGroup* groups, const unsigned char* active, const unsigned* flags,
+                              cudaStream_t st);
+// One phase on tiles of one or two 256-column blocks (NsTile::nh), bf16
+// operands; split_ws: non-NULL only for a Gram launch with split-K parts;
+// pdl: programmatic dependent launch (the kernel may start while the
+// previous kernel on the stream finishes).
+cudaError_t launch_ns_wide_phase(NsPhase ph, int iter, int ngroups, const NsGroup* groups, const TcGroupMaps* maps,
+                                 const NsTile* tiles, int ntiles, const int* offsets, int npairs,
+                                 const double* norm2, NsCoeffs co, unsigned* flags, const FuseFinal* fuse,
+                                 cudaStream_t st, const unsigned char* active, float* split_ws, bool pdl,
+                                 uint64_t wait_ns);
 // fp32 -> three bf16 planes (hi, mid, lo; their sum is exactly the input):
 // n elements of src, plane q at dst + q * n.
 cudaError_t launch_split3(const float* src, void* dst, size_t n, const unsigned* flags, cudaStream_t st);
-// After a Gram launch with split tiles: bf16 A tiles from the fp32 parts.
+// After a wide Gram launch with split tiles: bf16 A tiles from the fp32 parts.
 cudaError_t launch_ns_split_finish(const NsSplitTarget* targets, int n, const float* ws, const unsigned* flags,
                                    cudaStream_t st);
 

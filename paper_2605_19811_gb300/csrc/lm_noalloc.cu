@@ -22,6 +22,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include <cudaTypedefs.h>
 
@@ -102,6 +103,7 @@ struct BuildArgs {
   NsTile* d_tiles[3];
   int bm, bn;
   double* d_norm2;
+  uint32_t* d_done;
   unsigned* d_flags;
 };
 
@@ -112,6 +114,7 @@ __global__ void build_tables_kernel(BuildArgs a) {
     *a.d_mat = a.mat;
     *a.d_group = a.group;
     *a.d_norm2 = 0.0;
+    for (int ph = 0; ph < 3; ++ph) a.d_done[ph] = 0u;
     *a.d_flags = 0u;
   }
   const int64_t numel = a.mat.rows * a.mat.cols;
@@ -184,7 +187,9 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   const int s = (int)std::min(in->rows, in->cols), l = (int)std::max(in->rows, in->cols);
   const int s_pad = xdt == LM_BF16 ? tc_pad_s(s) : simt_pad(s);
   const int l_pad = xdt == LM_BF16 ? tc_pad_l(l) : simt_pad(l);
-  const int bm = xdt == LM_BF16 ? kTcBM : kSimtBM, bn = xdt == LM_BF16 ? kTcBN : kSimtBN;
+  const int bm = xdt == LM_BF16 ? kTcBM : kSimtBM;
+  const int bn = xdt == LM_BF16 ? tc_tile_cols(phase_tiles(NS_APPLY, s_pad, l_pad, in->rows > in->cols, bm, kTcBN), 1)
+                                : kSimtBN;
   const size_t es = xdt == LM_BF16 ? 2 : 4;
   const int tall = in->rows > in->cols ? 1 : 0;
   const int64_t numel = in->rows * in->cols;
@@ -194,7 +199,7 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
 
   size_t off = 0;
   const size_t off_flags = off;   off = align256(off + sizeof(unsigned));
-  const size_t off_norm = off;    off = align256(off + sizeof(double));
+  const size_t off_norm = off;    off = align256(off + sizeof(double) + 3 * sizeof(uint32_t));
   const size_t off_mat = off;     off = align256(off + sizeof(MatDesc));
   const size_t off_group = off;   off = align256(off + sizeof(NsGroup));
   const size_t off_et = off;      off = align256(off + (size_t)n_et * sizeof(ElemChunk));
@@ -230,6 +235,9 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   g.l_pad = l_pad;
   g.first_mat = 0;
   g.tall = tall;
+  g.n_gram = ntiles[NS_GRAM];
+  g.n_poly = ntiles[NS_POLY];
+  g.n_apply = ntiles[NS_APPLY];
   g.X[0] = base + off_x0;
   g.X[1] = base + off_x1;
   g.A = base + off_a;
@@ -260,11 +268,12 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   ba.bm = bm;
   ba.bn = bn;
   ba.d_norm2 = d.norm2;
+  ba.d_done = reinterpret_cast<uint32_t*>(d.norm2 + 1);
   ba.d_flags = reinterpret_cast<unsigned*>(base + off_flags);
 
   TcGroupMaps maps;
   if (xdt == LM_BF16) {
-    e = tc_encode_group_maps(g, &maps);
+    e = tc_encode_group_maps(g, &maps, 1, bn, false);
     if (e != cudaSuccess) return set_error(LM_ERR_CUDA, "cuTensorMapEncodeTiled failed");
   }
 
@@ -284,23 +293,34 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   e = launch_momentum_norm(xdt, in->dtype, ba.d_mat, ba.d_chunks, n_et, nullptr, mk, 1, stream);
   if (e != cudaSuccess) return set_error(LM_ERR_CUDA, cudaGetErrorString(e));
   const NsCoeffs co{(float)a, (float)b, (float)c, (float)eps};
-  // c = 0 (a cubic): B = b A is not formed, APPLY reads A and scales by b;
-  // otherwise, where |a| < 4, a is folded into B's diagonal (as lm_msign_ns
-  // does, unless LM_NS_FOLD=0)
-  const bool from_a = xdt == LM_BF16 && co.c == 0.f;
-  const char* fold_env = std::getenv("LM_NS_FOLD");
-  const bool fold = xdt == LM_BF16 && !from_a && std::fabs(co.a) < 4.f &&
-                    !(fold_env != nullptr && std::strcmp(fold_env, "0") == 0);
-  for (int it = 0; it < steps; ++it)
+  if (xdt == LM_BF16 && steps > 0) {
+    const std::vector<NsCoeffs> cos((size_t)steps, co);
+    const char* fold_env = std::getenv("LM_NS_FOLD");
+    NsChain ch{};
+    ch.ngroups = 1;
+    ch.groups = &g;
+    ch.maps = &maps;
     for (int ph = 0; ph < 3; ++ph) {
-      if (ph == NS_POLY && from_a) continue;
-      if (xdt == LM_BF16)
-        e = launch_ns_tc((NsPhase)ph, it, 1, &g, &maps, ba.d_tiles[ph], ntiles[ph], nullptr, 0,
-                         d.norm2, co, ba.d_flags, nullptr, stream, nullptr, nullptr, 1, 0, false, false,
-                         env_wait_limit_ns(), ph == NS_APPLY && from_a, ph != NS_GRAM && fold);
-      else
-        e = launch_ns_simt((NsPhase)ph, it, 1, ba.d_group, ba.d_tiles[ph], ntiles[ph], d.norm2, co,
-                           stream, nullptr, nullptr, ba.d_flags);
+      ch.tiles[ph] = ba.d_tiles[ph];
+      ch.ntiles[ph] = ntiles[ph];
+    }
+    ch.npairs = std::min(tc_max_pairs(), std::max(ntiles[0], std::max(ntiles[1], ntiles[2])));
+    ch.done = ba.d_done;
+    ch.norm2 = d.norm2;
+    ch.steps = steps;
+    ch.co = cos.data();
+    ch.fold = !(fold_env != nullptr && std::strcmp(fold_env, "0") == 0);
+    ch.pieces = 1;
+    ch.bn = bn;
+    ch.flags = ba.d_flags;
+    ch.wait_ns = env_wait_limit_ns();
+    e = launch_ns_chain(ch, 0, 3 * steps, stream);
+    if (e != cudaSuccess) return set_error(LM_ERR_CUDA, cudaGetErrorString(e));
+  }
+  for (int it = 0; it < steps && xdt == LM_F32; ++it)
+    for (int ph = 0; ph < 3; ++ph) {
+      e = launch_ns_simt((NsPhase)ph, it, 1, ba.d_group, ba.d_tiles[ph], ntiles[ph], d.norm2, co, stream, nullptr,
+                         nullptr, ba.d_flags);
       if (e != cudaSuccess) return set_error(LM_ERR_CUDA, cudaGetErrorString(e));
     }
   e = launch_finalize(xdt, out->dtype, ba.d_mat, ba.d_chunks, n_et, mk, 1, ba.d_flags, stream);

@@ -30,11 +30,7 @@ struct TcParams {
   FuseFinal fuse;       // fuse.mats != NULL: this APPLY writes the parameters
   const unsigned char* active;   // NULL, or per matrix: 0 = skip its tiles
   float* split_ws;               // fp32 workspace of split Gram tiles (256 x 256 each)
-  int final_f32;                 // three-piece operands: this APPLY writes fp32 X to NsGroup::Xf
   uint64_t wait_ns;              // limit of every bounded wait of the roles
-  int apply_from_a;              // APPLY of an iteration with c = 0: B = b A was not formed,
-                                 // the left operand is A and the accumulator is scaled by b
-  int fold_a;                    // POLY adds a to B's diagonal (B' = a I + B); APPLY is X' = B' X
 };
 
 // Launch of the wide-tile kernel (lm_ns_wide.cu); grid = 2 x CTA pairs.
@@ -73,6 +69,12 @@ static_assert(kThreads == 32 * (3 + kEpiWarps), "role layout");
 constexpr int kAuxBoxBytes = kHalf * 64 * 2;         // one 64-column box of the CTA's rows: 16 KB
 constexpr uint64_t kCleanupWaitNs = 100000000ull;    // waits for in-flight copies after a give-up
 
+// b v + c acc of the polynomial phase, in one order of roundings for both
+// kernels (left to the compiler, the contraction differs from loop to loop).
+__device__ __forceinline__ float poly_value(float b, float v, float c, float acc) {
+  return __fmaf_rn(b, v, __fmul_rn(c, acc));
+}
+
 // Whether a tile's matrix runs in this launch; every role asks the same
 // question of the same tiles, so skipping keeps their pipelines in step.
 __device__ __forceinline__ bool tile_active(const TcParams& p, const NsTile& t) {
@@ -85,10 +87,10 @@ __device__ __forceinline__ bool tile_active(const TcParams& p, const NsTile& t) 
 // bounded wait (LM_FLAG_TIMEOUT).  CTA 0 of the pair reads the status word
 // and CTA 1 takes CTA 0's answer, so both CTAs agree even if another pair
 // of this launch raises the flag meanwhile.
-__device__ __forceinline__ bool pair_start(const TcParams& p, uint32_t* stop_word, uint32_t rank) {
+__device__ __forceinline__ bool pair_start(const unsigned* flags, uint32_t* stop_word, uint32_t rank) {
   tc::griddep_wait();
   if (threadIdx.x == 0)
-    *stop_word = rank == 0 ? ((*reinterpret_cast<volatile unsigned*>(p.flags) & LM_FLAG_TIMEOUT) != 0u) : 0u;
+    *stop_word = rank == 0 ? ((*reinterpret_cast<const volatile unsigned*>(flags) & LM_FLAG_TIMEOUT) != 0u) : 0u;
   tc::tc_fence_before();
   tc::cluster_sync();   // barriers of both CTAs initialised, CTA 0's answer visible
   tc::tc_fence_after();

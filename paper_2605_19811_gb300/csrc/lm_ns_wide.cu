@@ -276,7 +276,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tmem_alloc(tmem_slot, kTmemColsW);
     tmem_relinquish();
   }
-  if (pair_start(p, stop_word, rank)) w_begin = w_end;   // an earlier launch gave up: no tiles
+  if (pair_start(p.flags, stop_word, rank)) w_begin = w_end;   // an earlier launch gave up: no tiles
   const uint32_t tmem_base = *tmem_slot;
   const uint64_t wait_ns = p.wait_ns;
 
@@ -502,7 +502,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               const float acc = __uint_as_float(r[e]);
               float o;
               if (phase == NS_GRAM) o = acc * nscale;
-              else if (phase == NS_POLY) o = p.co.b * v[e] + p.co.c * acc;
+              else if (phase == NS_POLY) o = poly_value(p.co.b, v[e], p.co.c, acc);
               else o = __fmaf_rn(p.co.a, v[e], acc) * nscale;   // the same rounding as ns_tc_kernel
               v[e] = (i_row < nrows && j0 + e < ncols) ? o : 0.f;
             }

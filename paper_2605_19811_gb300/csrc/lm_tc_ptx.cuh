@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "lionmuon.h"
+
 namespace lm {
 namespace tc {
 namespace {
@@ -48,9 +50,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 // Bounded wait for the phase with the given parity.  Returns false if the
 // time limit passed or another role asked to stop.  The first probe is
-// inlined; the slow path is a call.  It reads the clock every 256 probes, or
-// after every probe when the limit is under a millisecond (a short limit is a
-// failure test, and should give up at the first probe that finds nothing).
+// inlined; the slow path is a call.  Its probes suspend the thread for up to
+// kSuspendNs each (a waiting role then takes no issue slots and no power from
+// the MMAs) and it reads the clock every 8 of them, or after every probe when
+// the limit is under a millisecond (a short limit is a failure test, and should
+// give up at the first probe that finds nothing).
+constexpr uint32_t kSuspendNs = 20000;
 // The same probe with a suspend-time hint: the thread waits at most about
 // hint_ns inside the instruction.
 __device__ __forceinline__ bool mbar_try_wait_hint(uint64_t* bar, uint32_t parity, uint32_t hint_ns) {
@@ -68,9 +73,10 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, vola
                                             uint64_t limit_ns) {
   const uint64_t t0 = globaltimer();
   const bool short_limit = limit_ns < 1000000ull;
-  const uint32_t every = short_limit ? 0u : 255u;
+  const uint32_t every = short_limit ? 0u : 7u;
+  const uint32_t hint = short_limit ? (uint32_t)limit_ns : kSuspendNs;
   for (uint32_t i = 1;; ++i) {
-    if (short_limit ? mbar_try_wait_hint(bar, parity, (uint32_t)limit_ns) : mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait_hint(bar, parity, hint)) return true;
     if ((i & every) == 0) {
       if (*abort_flag) return false;
       if (globaltimer() - t0 > limit_ns) return false;
@@ -81,6 +87,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
                                           uint64_t limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, abort_flag, limit_ns);
+}
+// The same wait by a whole converged warp, with one answer for all lanes.  A
+// lane waiting for its warp (and a shuffle of the answer) costs the warp its
+// convergence: the shuffle took 1800 cycles more than the wait.
+__device__ __noinline__ bool mbar_wait_warp_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                 uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  const bool short_limit = limit_ns < 1000000ull;
+  const uint32_t every = short_limit ? 0u : 7u;
+  const uint32_t hint = short_limit ? (uint32_t)limit_ns : kSuspendNs;
+  for (uint32_t i = 1;; ++i) {
+    const bool ok = mbar_try_wait_hint(bar, parity, hint);
+    if (__any_sync(0xffffffffu, ok)) return true;
+    if ((i & every) == 0 && __any_sync(0xffffffffu, *abort_flag != 0 || globaltimer() - t0 > limit_ns)) return false;
+  }
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               uint64_t limit_ns) {
+  if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return mbar_wait_warp_slow(bar, parity, abort_flag, limit_ns);
 }
 // 3-D tiled TMA load into this CTA's shared memory; completion is signalled
 // on the mbarrier at shared::cluster address bar_cluster (either CTA of the pair).
@@ -124,6 +150,10 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void*
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+template <int kPending>
+__device__ __forceinline__ void bulk_wait_read() {   // all but the last kPending groups have read their source
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kPending) : "memory");
 }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Make this thread's generic-proxy shared-memory writes visible to the TMA.
@@ -206,6 +236,36 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// The same load without its wait, and the wait: the registers may be used
+// only after tmem_ld_wait on them.
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32"
+      " {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15,"
+      " %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31},"
+      " [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
+}
+// 32-byte global store of eight floats (p 32-byte aligned).
+__device__ __forceinline__ void st_global_v8(float* p, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
 // Shared-memory matrix descriptor (tcgen05), 128-byte swizzle.
 //   bits 0-13  start address >> 4
 //   bits 16-29 leading-dimension byte offset >> 4
@@ -237,6 +297,73 @@ __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 
 __device__ __forceinline__ uint32_t pack_bf2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// Counters in global memory that order tiles of one launch (the chain kernel):
+// a producer of data makes it visible and adds with release, a consumer polls
+// with acquire.  Data that goes through the async proxy (TMA) on either side
+// also needs the proxy fence there.
+__device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release_gpu(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Orders this thread's earlier (acquired) view of global memory before its
+// later TMA copies.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+// Bounded wait until the counter has reached `target` (counters only grow).
+// Returns false when the limit passed, another role of this CTA asked to stop
+// or another CTA recorded a give-up in *flags.
+__device__ __noinline__ bool counter_wait_slow(const uint32_t* ctr, uint32_t target, const unsigned* flags,
+                                               volatile int* abort_flag, uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  const uint32_t every = limit_ns < 1000000ull ? 0u : 63u;
+  for (uint32_t i = 1;; ++i) {
+    if ((int32_t)(ld_acquire_gpu(ctr) - target) >= 0) return true;
+    __nanosleep(64);
+    if ((i & every) == 0) {
+      if (*abort_flag) return false;
+      if (*reinterpret_cast<const volatile unsigned*>(flags) & LM_FLAG_TIMEOUT) return false;
+      if (globaltimer() - t0 > limit_ns) return false;
+    }
+  }
+}
+__device__ __forceinline__ bool counter_wait(const uint32_t* ctr, uint32_t target, const unsigned* flags,
+                                             volatile int* abort_flag, uint64_t limit_ns) {
+  if ((int32_t)(ld_acquire_gpu(ctr) - target) >= 0) return true;
+  return counter_wait_slow(ctr, target, flags, abort_flag, limit_ns);
+}
+
+// A counter in this CTA's shared memory: add with release, and a bounded
+// wait (acquire) until it has reached `target`.
+__device__ __forceinline__ void smem_counter_add(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.cta.shared::cta.add.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_counter_read(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __noinline__ bool smem_counter_wait_slow(const uint32_t* p, uint32_t target, volatile int* abort_flag,
+                                                    uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  const uint32_t every = limit_ns < 1000000ull ? 0u : 63u;
+  for (uint32_t i = 1;; ++i) {
+    __nanosleep(20);
+    if ((int32_t)(smem_counter_read(p) - target) >= 0) return true;
+    if ((i & every) == 0) {
+      if (*abort_flag) return false;
+      if (globaltimer() - t0 > limit_ns) return false;
+    }
+  }
+}
+__device__ __forceinline__ bool smem_counter_wait(const uint32_t* p, uint32_t target, volatile int* abort_flag,
+                                                  uint64_t limit_ns) {
+  if ((int32_t)(smem_counter_read(p) - target) >= 0) return true;
+  return smem_counter_wait_slow(p, target, abort_flag, limit_ns);
 }
 
 // Programmatic dependent launch: wait until the grid this launch depends on
