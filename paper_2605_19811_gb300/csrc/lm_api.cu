@@ -256,7 +256,12 @@ static std::atomic<bool> g_nvtx{false};
 static const char* const kFamilyNames[LM_KERNEL_FAMILIES] = {
     "lion", "momentum_norm", "ns_gram", "ns_poly", "ns_apply", "finalize", "other", "adamw", "srank"};
 
-constexpr int64_t kLionChunk = 32768;   // elements per Lion work chunk
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
 // Three-piece mode: Gram tiles longer than this many 64-deep K blocks (1536)
 // are split along K, whatever the balance (the parts are added in fp32): the
 // tensor cores' fp32 accumulation error grows with the MMAs summed into one
@@ -297,13 +302,16 @@ struct AdamTable {
 
 template <typename TensorT>
 void build_lion_chunks(const std::vector<TensorT>& ts, std::vector<LionChunk>& out) {
+  int64_t total = 0;
+  for (const TensorT& t : ts) total += t.n;
+  const int64_t chunk = elem_chunk(total, sm_count());
   for (size_t i = 0; i < ts.size(); ++i) {
-    for (int64_t b = 0; b < ts[i].n; b += kLionChunk) {
+    for (int64_t b = 0; b < ts[i].n; b += chunk) {
       LionChunk c;
       c.tensor = (int32_t)i;
       c.pad = 0;
       c.begin = b;
-      c.count = std::min<int64_t>(kLionChunk, ts[i].n - b);
+      c.count = std::min<int64_t>(chunk, ts[i].n - b);
       out.push_back(c);
     }
   }
@@ -373,12 +381,15 @@ void build_ns_tiles(const std::vector<NsGroup>& groups, int g0, int ng, int phas
   for (auto& e : v) out.push_back(e.second);
 }
 
-// Element chunks of each matrix (kElemChunk elements, the last one ragged).
+// Element chunks of each matrix (elem_chunk elements, the last one ragged).
 void build_elem_chunks(const std::vector<MatDesc>& mats, std::vector<ElemChunk>& out) {
+  int64_t total = 0;
+  for (const MatDesc& d : mats) total += d.rows * d.cols;
+  const int64_t chunk = elem_chunk(total, sm_count());
   for (size_t i = 0; i < mats.size(); ++i) {
     const int64_t n = mats[i].rows * mats[i].cols;
-    for (int64_t b = 0; b < n; b += kElemChunk)
-      out.push_back(ElemChunk{(int32_t)i, 0, b, std::min<int64_t>(kElemChunk, n - b)});
+    for (int64_t b = 0; b < n; b += chunk)
+      out.push_back(ElemChunk{(int32_t)i, 0, b, std::min<int64_t>(chunk, n - b)});
   }
 }
 

@@ -2,8 +2,8 @@
 //   * lion_kernel           : Lion branch + momentum update, multi-tensor,
 //                             one pass over W, G, M with 16-byte vector I/O.
 //   * momentum_norm_kernel  : Muon steps, first part: G_hat, ||G_hat||_F^2
-//                             (warp shuffle, one fp64 atomic per warp and
-//                             32K-element chunk), M update, X0 = G_hat.
+//                             (one fp64 atomic per chunk), M update,
+//                             X0 = G_hat.
 //   * finalize_kernel       : Muon steps, last part: W <- W - eta_M (0.2
 //                             sqrt(max(m,n)) X_K + lambda W) (Table 5 scaling),
 //                             or the plain msign output.
@@ -228,6 +228,52 @@ __device__ __forceinline__ int64_t x_index(const MatDesc& d, int64_t e) {
   return r * d.ldx + (e - r * d.cols);
 }
 
+// Eight consecutive elements e .. e + 7 of a matrix whose row length is not a
+// multiple of 8, in X: they may span rows, and a row starts at any offset of a
+// vector, so they move in units of 4, 2 or 1 elements, the largest that divides
+// the row length (a unit then never spans rows and is aligned in X, whose pitch
+// is a multiple of 128).  G, M and W are contiguous and keep their 16-byte
+// vectors.  One element per thread and trip, the form before, took 84 us
+// (momentum + norm) and 87 us (finalize) for 4.77 M elements with rows of
+// 300, 900 and 1200; with these they take 16 and 13 us (ncu, cold cache).
+template <int U, typename T>
+struct UnitVec {
+  struct alignas(U * sizeof(T)) type {
+    T v[U];
+  };
+};
+template <int U, typename T>
+__device__ __forceinline__ void x_units(const MatDesc& d, T* x, int64_t e, float (&v)[8], bool store) {
+  using Vec = typename UnitVec<U, T>::type;
+  int64_t r = e < 0xFFFFFFFFll && d.cols < 0xFFFFFFFFll ? (int64_t)((uint32_t)e / (uint32_t)d.cols) : e / d.cols;
+  int64_t c = e - r * d.cols;
+#pragma unroll
+  for (int k = 0; k < 8 / U; ++k) {
+    while (c >= d.cols) {
+      c -= d.cols;
+      ++r;
+    }
+    Vec* p = reinterpret_cast<Vec*>(x + r * d.ldx + c);
+    if (store) {
+      Vec w;
+#pragma unroll
+      for (int j = 0; j < U; ++j) w.v[j] = from_f<T>(v[k * U + j]);
+      *p = w;
+    } else {
+      const Vec w = *p;
+#pragma unroll
+      for (int j = 0; j < U; ++j) v[k * U + j] = to_f(w.v[j]);
+    }
+    c += U;
+  }
+}
+template <typename T>
+__device__ __forceinline__ void x_ragged(const MatDesc& d, T* x, int64_t e, float (&v)[8], bool store) {
+  if ((d.cols & 3) == 0) x_units<4>(d, x, e, v, store);
+  else if ((d.cols & 1) == 0) x_units<2>(d, x, e, v, store);
+  else x_units<1>(d, x, e, v, store);
+}
+
 // Muon direction for 8 elements: G_hat = b1 M + c1 G (fp32, same operation
 // order as the Lion step), M <- b2 M + c2 G; returns sum G_hat^2.
 __device__ __forceinline__ float momentum_math(float (&gv)[8], float (&mv)[8], float (&gh)[8],
@@ -251,10 +297,25 @@ __device__ __forceinline__ float momentum_math(float (&gv)[8], float (&mv)[8], f
 constexpr int kMomVec = 3, kMomCtas = 2;
 constexpr int kFinVec = 2, kFinCtas = 3;
 
+// A thread's sum of squares: each vector's 8 squares are summed in fp32, the
+// vectors with the rounding error of every addition carried along (Knuth's
+// two-sum), so the norm does not depend on how elements fall into chunks (ranks
+// of a sharded set chunk differently) and costs no fp64 arithmetic per vector
+// (this GPU's fp64 rate is a small fraction of its fp32 rate).
+struct SquareSum {
+  float s = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float a) {
+    const float t = __fadd_rn(s, a);
+    const float b = __fsub_rn(t, s);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b)));
+    s = t;
+  }
+};
+
 template <typename XT, typename GT>
-__device__ float momentum_chunk(const MatDesc& d, int64_t begin, int64_t count, const GT* g,
-                                const MuonConsts& k, int mode) {
-  float acc = 0.f;
+__device__ SquareSum momentum_chunk(const MatDesc& d, int64_t begin, int64_t count, const GT* g,
+                                    const MuonConsts& k, int mode) {
+  SquareSum acc;
   XT* x = static_cast<XT*>(d.x);
   if ((d.cols & 7) == 0) {
     // rows hold whole vectors; count is a multiple of 8.  kMomVec vectors
@@ -270,7 +331,7 @@ __device__ float momentum_chunk(const MatDesc& d, int64_t begin, int64_t count, 
         if (mode == 0) load8(d.m + e, mv[u]);
       }
 #pragma unroll
-      for (int u = 0; u < kMomVec; ++u) acc += momentum_math(gv[u], mv[u], hv[u], k, mode);
+      for (int u = 0; u < kMomVec; ++u) acc.add(momentum_math(gv[u], mv[u], hv[u], k, mode));
 #pragma unroll
       for (int u = 0; u < kMomVec; ++u) {
         const int64_t e = begin + (v + u * kElemThreads) * 8;
@@ -283,12 +344,22 @@ __device__ float momentum_chunk(const MatDesc& d, int64_t begin, int64_t count, 
       float ga[8], ma[8], ha[8];
       load8(g + ea, ga);
       if (mode == 0) load8(d.m + ea, ma);
-      acc += momentum_math(ga, ma, ha, k, mode);
+      acc.add(momentum_math(ga, ma, ha, k, mode));
       if (mode == 0) store8(d.m + ea, ma);
       store8(x + x_index(d, ea), ha);
     }
   } else {
-    for (int64_t e = begin + threadIdx.x; e < begin + count; e += kElemThreads) {
+    const int64_t nvec = count >> 3;
+    for (int64_t v = threadIdx.x; v < nvec; v += kElemThreads) {
+      const int64_t e = begin + v * 8;
+      float gv[8], mv[8], hv[8];
+      load8(g + e, gv);
+      if (mode == 0) load8(d.m + e, mv);
+      acc.add(momentum_math(gv, mv, hv, k, mode));
+      if (mode == 0) store8(d.m + e, mv);
+      x_ragged(d, x, e, hv, true);
+    }
+    for (int64_t e = begin + (nvec << 3) + threadIdx.x; e < begin + count; e += kElemThreads) {   // a matrix's last elements
       const float gv = to_f(g[e]);
       float gh = gv;
       if (mode == 0) {
@@ -296,7 +367,7 @@ __device__ float momentum_chunk(const MatDesc& d, int64_t begin, int64_t count, 
         gh = __fadd_rn(__fmul_rn(k.b1, mv), __fmul_rn(k.c1, gv));
         d.m[e] = __fadd_rn(__fmul_rn(k.b2, mv), __fmul_rn(k.c2, gv));
       }
-      acc = fmaf(gh, gh, acc);
+      acc.add(__fmul_rn(gh, gh));
       x[x_index(d, e)] = from_f<XT>(gh);
     }
   }
@@ -307,6 +378,7 @@ template <typename XT, typename GT, int MODE>
 __global__ void __launch_bounds__(kElemThreads, kMomCtas)
     momentum_norm_kernel(const MatDesc* __restrict__ mats, const ElemChunk* __restrict__ chunks,
                          int nchunks, const void* const* __restrict__ grads, MuonConsts k) {
+  __shared__ double part[kElemThreads / 32];
   if (lm_stopped(k.flags)) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
@@ -314,11 +386,20 @@ __global__ void __launch_bounds__(kElemThreads, kMomCtas)
     if (k.active != nullptr && !k.active[ch.mat]) continue;   // this matrix takes the Lion step
     const MatDesc& d = mats[ch.mat];
     const GT* src = static_cast<const GT*>(MODE == 0 ? grads[d.grad_slot] : d.w);
-    float acc = momentum_chunk<XT>(d, ch.begin, ch.count, src, k, MODE);
-    // ||G_hat||_F^2: warp shuffle, then one fp64 atomic per warp and chunk
+    const SquareSum acc = momentum_chunk<XT>(d, ch.begin, ch.count, src, k, MODE);
+    // ||G_hat||_F^2: warp shuffle and shared memory, one fp64 atomic per chunk
+    double sum = (double)acc.s + (double)acc.lo;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(d.norm2, (double)acc);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double all = 0.0;
+#pragma unroll
+      for (int w = 0; w < kElemThreads / 32; ++w) all += part[w];
+      atomicAdd(d.norm2, all);
+    }
+    __syncthreads();   // part is reused by the next chunk
   }
 }
 
@@ -365,7 +446,16 @@ __device__ void finalize_chunk(const MatDesc& d, int64_t begin, int64_t count, c
       store8(p + ea, pa);
     }
   } else {
-    for (int64_t e = begin + threadIdx.x; e < begin + count; e += kElemThreads) {
+    const int64_t nvec = count >> 3;
+    for (int64_t v = threadIdx.x; v < nvec; v += kElemThreads) {
+      const int64_t e = begin + v * 8;
+      float xv[8], pv[8];
+      x_ragged(d, const_cast<XT*>(x), e, xv, false);
+      if (mode == 0) load8(p + e, pv);
+      finalize_math(xv, pv, d.shape_scale, k, mode, xs, scale_x);
+      store8(p + e, pv);
+    }
+    for (int64_t e = begin + (nvec << 3) + threadIdx.x; e < begin + count; e += kElemThreads) {
       float xv = to_f(x[x_index(d, e)]);
       if (scale_x) xv = __fmul_rn(xv, xs);
       float pv = mode == 0 ? to_f(p[e]) : 0.f;

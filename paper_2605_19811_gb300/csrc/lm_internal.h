@@ -100,7 +100,17 @@ struct ElemChunk {
   int64_t begin;
   int64_t count;
 };
-constexpr int64_t kElemChunk = 32768;   // elements per chunk
+// Elements per chunk of an element-wise kernel: 32768, less for sets so small
+// that such chunks would leave SMs without work (about two chunks per resident
+// block, two blocks per SM, in steps of one 8-element vector per thread).  Tiny
+// set (0.66 M elements, 320 chunks for 20): momentum + norm 14.5 -> 9.8 us,
+// finalize 12.7 -> 7.0 us (ncu, cold cache).
+constexpr int64_t kElemChunk = 32768;
+inline int64_t elem_chunk(int64_t total, int sms) {
+  const int64_t per = total / (4 * (int64_t)(sms > 0 ? sms : 1));
+  const int64_t c = (per + 2047) / 2048 * 2048;
+  return c < 2048 ? 2048 : (c > kElemChunk ? kElemChunk : c);
+}
 struct MuonConsts {
   float b1, c1, b2, c2;   // interpolation / momentum constants
   float eM, lam;          // Muon learning rate and weight decay

@@ -100,6 +100,7 @@ struct BuildArgs {
   NsGroup* d_group;
   ElemChunk* d_chunks;
   int n_chunks;
+  int64_t chunk;
   NsTile* d_tiles[3];
   int bm, bn;
   double* d_norm2;
@@ -119,8 +120,8 @@ __global__ void build_tables_kernel(BuildArgs a) {
   }
   const int64_t numel = a.mat.rows * a.mat.cols;
   for (int i = threadIdx.x; i < a.n_chunks; i += blockDim.x) {
-    const int64_t b = (int64_t)i * kElemChunk;
-    a.d_chunks[i] = ElemChunk{0, 0, b, numel - b < kElemChunk ? numel - b : kElemChunk};
+    const int64_t b = (int64_t)i * a.chunk;
+    a.d_chunks[i] = ElemChunk{0, 0, b, numel - b < a.chunk ? numel - b : a.chunk};
   }
   if (threadIdx.x < 3) {
     const int ph = threadIdx.x;
@@ -193,7 +194,6 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   const size_t es = xdt == LM_BF16 ? 2 : 4;
   const int tall = in->rows > in->cols ? 1 : 0;
   const int64_t numel = in->rows * in->cols;
-  const int n_et = (int)((numel + kElemChunk - 1) / kElemChunk);
   int ntiles[3];
   for (int ph = 0; ph < 3; ++ph) ntiles[ph] = phase_tiles(ph, s_pad, l_pad, tall, bm, bn);
 
@@ -202,7 +202,6 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   const size_t off_norm = off;    off = align256(off + sizeof(double) + 3 * sizeof(uint32_t));
   const size_t off_mat = off;     off = align256(off + sizeof(MatDesc));
   const size_t off_group = off;   off = align256(off + sizeof(NsGroup));
-  const size_t off_et = off;      off = align256(off + (size_t)n_et * sizeof(ElemChunk));
   size_t off_tiles[3];
   for (int ph = 0; ph < 3; ++ph) {
     off_tiles[ph] = off;
@@ -213,6 +212,13 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   const size_t off_x1 = off;  off = align256(off + xbytes);
   const size_t off_a = off;   off = align256(off + abytes);
   const size_t off_b = off;   off = align256(off + abytes);
+  // the element chunks come last: short ones where their table still fits
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int64_t chunk = elem_chunk(numel, sms);
+  if (off + (size_t)((numel + chunk - 1) / chunk) * sizeof(ElemChunk) > kNoAllocScratchBytes) chunk = kElemChunk;
+  const int n_et = (int)((numel + chunk - 1) / chunk);
+  const size_t off_et = off;  off = align256(off + (size_t)n_et * sizeof(ElemChunk));
   if (off > kNoAllocScratchBytes) {
     char msg[256];
     snprintf(msg, sizeof(msg),
@@ -264,6 +270,7 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   ba.d_group = reinterpret_cast<NsGroup*>(base + off_group);
   ba.d_chunks = reinterpret_cast<ElemChunk*>(base + off_et);
   ba.n_chunks = n_et;
+  ba.chunk = chunk;
   for (int ph = 0; ph < 3; ++ph) ba.d_tiles[ph] = reinterpret_cast<NsTile*>(base + off_tiles[ph]);
   ba.bm = bm;
   ba.bn = bn;

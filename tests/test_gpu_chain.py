@@ -75,3 +75,46 @@ def test_one_launch_equals_one_launch_per_phase(shapes, cfg, precision, dtype):
     b = _steps(shapes, True, dtype=dtype, ns_precision=precision, **cfg)
     for x, y in zip(a, b):
         np.testing.assert_array_equal(x, y)
+
+
+# Element-wise kernels around the Newton-Schulz chain: row lengths that take
+# units of 4, 2 and 1 elements and rows shorter than a vector, counts that are
+# and are not multiples of 8 (the last elements), and a set small enough for
+# short chunks next to one with whole chunks
+@pytest.mark.parametrize("shape", [(37, 300), (300, 36), (64, 1202), (33, 301), (257, 5), (5, 3), (1201, 2), (2, 4099),
+                                   (1000, 1301)])
+@pytest.mark.parametrize("dtype,precision", [("bf16", 1), ("f32", 1), ("f32", 0), ("bf16", 0)])
+def test_ragged_rows_step(shape, dtype, precision):
+    """A Muon step against the storage-modelled oracle: momentum bit-exact,
+    W <- W - eta (s NS(G_hat) + lambda W) within the NS tolerance."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    w0 = host_tensor(synth.init_weights([shape], seed=2)[0], dtype)
+    g = host_tensor(synth.draw_matrix(shape, seed=7), dtype)
+    p = w0.cuda()
+    opt = L.LionMuon([p], period=1, eta_muon=0.02, weight_decay=0.1, ns_precision=precision)
+    opt.step([g.cuda()], 0)
+    torch.cuda.synchronize()
+    assert opt.status() == 0
+    m = (np.float32(1.0 - 0.99) * g.float().numpy()).astype(np.float32)
+    np.testing.assert_array_equal(bits(opt.momentum(0)), m.view(np.uint32))
+    gh = (np.float32(1.0 - 0.9) * g.float().numpy()).astype(np.float32).astype(np.float64)
+    x = host_tensor(gh, "bf16") if precision == 1 else gh
+    ns = ns_closed_form_rows(stored_values(x) if precision == 1 else x, 5, *QUINTIC, 1e-7)
+    ns = ns if shape[0] >= shape[1] else ns.T
+    upd = 0.02 * 0.2 * np.sqrt(max(shape)) * ns
+    w = stored_values(w0)
+    want = w - upd - 0.02 * 0.1 * w
+    # the NS tolerance (2e-2 bf16, 1e-5 fp32), or 1.5 times what keeping X, A
+    # and B in the path's storage type does to this input by itself (the
+    # storage-modelled oracle; 2.1e-2 in bf16 on the 37 x 300 one)
+    table = (QUINTIC,) * 5
+    d = rel_fro(O.ns_polynomial_schedule_storage(gh, table, 1e-7, "bf16" if precision == 1 else "f32"),
+                O.ns_polynomial_schedule(gh, table, 1e-7))
+    tau = max(2e-2 if precision == 1 else 1e-5, 1.5 * d)
+    # the NS tolerance of the update, and half a unit in the last place of W's
+    # type per entry (2^-9 bf16, 2^-24 fp32)
+    ulp = 2.0 ** -9 if dtype == "bf16" else 2.0 ** -24
+    bound = tau * np.linalg.norm(upd) + 2 * ulp * np.linalg.norm(want)
+    assert np.linalg.norm(stored_values(p) - want) <= bound
+    opt.close()
