@@ -79,7 +79,10 @@ typedef struct {
  *   LM_NVTX=1           NVTX ranges named after the kernel families around the
  *                       library's launches
  *   LM_FAULT=oom        lm_create returns LM_ERR_OOM as if the device allocation
- *                       had failed (to exercise callers' error paths)
+ *                       had failed (to exercise callers' error paths);
+ *                       LM_FAULT=oom_f32tc: only the allocation with the
+ *                       three-piece workspace of LM_F32 fails, so that lm_create
+ *                       falls back to the CUDA-core path
  *   LM_NS_FORCE_FP32=1  the fp32 Newton-Schulz path whatever ns_precision says
  *   LM_NS_TILES=wide    bf16 Newton-Schulz tiles of two 256-column blocks per
  *                       CTA pair (the default is one block); same results bit
@@ -104,11 +107,15 @@ typedef struct {
  * beta1, beta2 in [0, 1); eta_* >= 0; weight_decay >= 0;
  * period >= 1, or 0 for P = infinity (never Muon);
  * ns_steps in [0, 64]; ns_eps >= 0; shape_scale >= 0;
- * ns_precision LM_BF16 (tensor-core bf16 GEMMs, fp32 accumulate), LM_F32
- * (fp32 CUDA-core GEMMs) or LM_NS_F32_TC (fp32 values on the tensor cores:
- * each fp32 operand is stored exactly as three bf16 pieces hi + mid + lo and
- * a product sums the six piece products down to order 2^-16, accumulated in
- * fp32; the fast fp32 mode, at the cost of six bf16 products per product).
+ * ns_precision LM_BF16 (tensor-core bf16 GEMMs, fp32 accumulate), LM_NS_F32_TC
+ * (fp32 values on the tensor cores: each fp32 operand is stored exactly as
+ * three bf16 pieces hi + mid + lo and a product sums the six piece products
+ * down to order 2^-16, accumulated in fp32; the fast fp32 mode, at the cost of
+ * six bf16 products per product) or LM_F32 (the exact fp32 mode: fp32 FMA on
+ * the CUDA cores, or, where every matrix has at least 320 rows and columns (256
+ * when every |a_k| < 4) and the workspace fits, the three pieces with their
+ * main products summed in fp32 registers per 64-deep block, which is closer to
+ * the fp64 iteration than the FMAs).
  * ns_coeffs: NULL for the same (ns_a, ns_b, ns_c) in every NS iteration, or
  * 3 * ns_steps finite values (a_k, b_k, c_k), k = 0 .. ns_steps - 1, for
  * iteration-dependent odd polynomials X <- a_k X + (b_k A + c_k A^2) X, the
@@ -271,9 +278,7 @@ lm_status lm_set_second_moment(lm_state* s, int i, const lm_tensor* src,
  * coefficients (a, b, c), normalisation X / (||X||_F + eps), iterated on the
  * wide orientation, with no 0.2 sqrt(max(m,n)) scaling.  in and out are
  * device tensors of equal shape (rows, cols >= 2 each), dtype LM_BF16 or
- * LM_F32 (may differ).  precision LM_BF16 uses the tensor-core path, LM_F32
- * the fp32 CUDA-core path, LM_NS_F32_TC fp32 values on the tensor cores (as
- * for lm_config::ns_precision).  Allocates its workspace with stream-ordered
+ * LM_F32 (may differ).  precision as lm_config::ns_precision.  Allocates its workspace with stream-ordered
  * allocation on cuda_stream and frees it the same way.  A testing entry
  * point: it synchronises cuda_stream before it returns, to read its own
  * status word.

@@ -201,9 +201,9 @@ MuonConsts muon_consts(const lm_config& c) {
 }
 
 // Device-memory arena: one cudaMalloc, sub-allocated with 256-byte alignment.
-// An allocation is laid out by two arenas: the tables (small, built on the
-// host and copied whole) and behind them the buffers (momentum, X, A, B, ...:
-// gigabytes that only start at zero, so the device clears them; copying them
+// An allocation is laid out by two arenas: the buffers (momentum, X, A, B, ...:
+// gigabytes that only start at zero, so the device clears them) and behind them
+// the tables (small, built on the host and copied whole).  Copying all of it
 // from a zeroed host image cost 4.1 of the 4.4 ms of a bf16 msign of a
 // 1280 x 5120 matrix, and seconds in lm_create of the 720M-shaped set).
 // With guard bands on (LM_DEBUG=1 when the state is created), every part is
@@ -232,7 +232,8 @@ struct Arena {
 // call starts; host side only, none of them changes the device code):
 //   LM_DEBUG=1         guard bands around every workspace part
 //   LM_NVTX=1          NVTX ranges around every kernel family's launches
-//   LM_FAULT=oom       lm_create fails with LM_ERR_OOM as if the allocation had
+//   LM_FAULT=oom       lm_create fails with LM_ERR_OOM as if the allocation had;
+//                      oom_f32tc: only with the three-piece workspace of LM_F32
 //   LM_NS_FORCE_FP32=1 the fp32 Newton-Schulz path whatever ns_precision says
 //   LM_NS_TILES=wide   two-block (256 x 512) Newton-Schulz tiles wherever
 //                      they fit, run by the wide-tile kernel; the default
@@ -286,6 +287,7 @@ struct NsBatch {
   int* offsets[3] = {nullptr, nullptr, nullptr};   // per-pair tile ranges (tensor-core path), NULL: snake order
   int npairs = 0;                                  // CTA pairs (tensor-core path)
   int bn = kTcBN;                                  // columns of a tile (tensor-core path)
+  int simt_tile[3] = {kSimtBM, kSimtBM, kSimtBM};  // tile of each phase (fp32 path)
   NsTile* compact[3] = {nullptr, nullptr, nullptr};   // masked steps: the selected matrices' tiles and their counts
   int* counts = nullptr;
   NsSplitTarget* split_targets = nullptr;   // split Gram tiles of this batch
@@ -403,6 +405,7 @@ lm_status set_error(lm_status st, const char* msg) { return fail(st, "%s", msg);
 struct NsEngine {
   lm_dtype xdt = LM_BF16;            // workspace dtype: bf16 (tensor cores) or fp32
   int pieces = 1;                    // tensor cores: 3 = fp32 values as three bf16 planes
+  bool promote = false;              // three pieces: the full-fp32 mode (LM_F32)
   std::vector<NsGroup> groups;       // host copies (device pointers inside)
   std::vector<TcGroupMaps> maps;     // tensor-core path
   NsGroup* d_groups = nullptr;       // device copy (fp32 path, tile compaction)
@@ -471,6 +474,7 @@ struct NsLayout {
   size_t off_groups = 0;
   size_t off_clear = 0;
   int nmat = 0, ntargets = 0;               // of the whole engine
+  int simt_parts = 0;                       // fp32 path: split-K parts of the phase that has most
   // split Gram tiles, per batch: (group, mat, tm, tn, first part, parts) of each target tile
   std::vector<std::vector<std::array<int, 6>>> split_targets;
   std::vector<size_t> off_split_targets;
@@ -558,8 +562,68 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
   t.swap(out);
 }
 
+// fp32 path: cuts the tiles of a phase along K where they leave resident
+// blocks without work: the shortest parts of at least 4 slices that leave at
+// most one part or tile per block; beside much longer tiles (a long-K embedding
+// Gram next to short hidden matrices, which would set the length of the
+// launch), tiles longer than twice a block's share into parts of half of it.
+// Returns the number of parts.
+static int split_simt_tiles(const std::vector<NsGroup>& groups, int g0, int phase, int tile, std::vector<NsTile>& t) {
+  const int slice = simt_slice(tile), blocks = simt_blocks(tile, sm_count());
+  auto len = [&](const NsTile& x) {
+    const NsGroup& g = groups[g0 + x.group];
+    return (int64_t)((phase == NS_GRAM ? g.l_pad : g.s_pad) / slice);
+  };
+  int64_t total = 0, longest = 0;
+  for (const NsTile& x : t) {
+    total += len(x);
+    longest = std::max(longest, len(x));
+  }
+  const int64_t avg = total / blocks;
+  int64_t part = 0;
+  if ((int64_t)t.size() < blocks) {
+    for (part = 4; part < longest; ++part) {
+      int64_t n = 0;
+      for (const NsTile& x : t) n += (len(x) + part - 1) / part;
+      if (n <= blocks) break;
+    }
+  } else if (longest > 2 * avg) {
+    part = std::max<int64_t>(8, avg / 2);
+  } else {
+    return 0;
+  }
+  const int64_t keep = (int64_t)t.size() < blocks ? part : 2 * avg;
+  std::vector<std::pair<int64_t, NsTile>> out;
+  int nparts_total = 0;
+  for (const NsTile& x : t) {
+    const int64_t nk = len(x);
+    const int n = (int)std::min<int64_t>(64, (nk + part - 1) / part);
+    if (nk <= keep || n < 2 || nparts_total + n > 65535) {
+      out.push_back({nk, x});
+      continue;
+    }
+    for (int k = 0; k < n; ++k) {
+      NsTile y = x;
+      y.kb0 = (uint16_t)(nk * k / n);
+      y.kb1 = (uint16_t)(nk * (k + 1) / n);
+      y.slot = (uint16_t)(nparts_total + k + 1);
+      y.nh = (uint16_t)(k << 8 | n);
+      out.push_back({y.kb1 - y.kb0, y});
+    }
+    nparts_total += n;
+  }
+  // longest first: blocks take tiles round robin
+  std::stable_sort(out.begin(), out.end(), [](const std::pair<int64_t, NsTile>& a, const std::pair<int64_t, NsTile>& c) {
+    return a.first > c.first;
+  });
+  t.clear();
+  for (const auto& x : out) t.push_back(x.second);
+  return nparts_total;
+}
+
 // Bytes of the block cleared at the start of a step: per matrix the norm
-// accumulator and three tile counters, per split target one counter.
+// accumulator and three tile counters, per split target (fp32 path: per part of
+// the phase that has most) one counter.
 static size_t ns_clear_bytes(int nmat, int ntargets) {
   return (size_t)nmat * (sizeof(double) + 3 * sizeof(uint32_t)) + (size_t)ntargets * sizeof(uint32_t);
 }
@@ -581,7 +645,7 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
     L.off_xf.push_back(pieces == 3 ? buf.add((size_t)g.count * g.s_pad * g.l_pad * sizeof(float)) : 0);
   }
   const int per = (xdt == LM_BF16) ? kMaxGroupsTc : kMaxGroupsSimt;
-  int max_split = 0;
+  size_t split_floats = 0;   // workspace of the split-K parts
   const int bm = (xdt == LM_BF16) ? kTcBM : kSimtBM;
   for (int g0 = 0; g0 < (int)groups.size(); g0 += per) {
     NsBatch b;
@@ -599,23 +663,30 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
         apply_tiles += (int64_t)groups[gi].count * ((groups[gi].s_pad + kTcBM - 1) / kTcBM) * (groups[gi].l_pad / kTcBN);
       b.bn = b.wide || !narrow_ok ? kTcBN : tc_tile_cols((int)std::min<int64_t>(apply_tiles, 1 << 30), pieces);
     }
-    const int bn = (xdt == LM_BF16) ? b.bn : kSimtBN;
+    const int bn = (xdt == LM_BF16) ? b.bn : kSimtBM;
     std::vector<NsTile> lists[3];
     std::vector<std::array<int, 6>> targets;
-    for (int ph = 0; ph < 3; ++ph) build_ns_tiles(groups, g0, b.ng, ph, bm, bn, lists[ph], b.wide);
+    for (int ph = 0; ph < 3; ++ph) {
+      build_ns_tiles(groups, g0, b.ng, ph, bm, bn, lists[ph], b.wide);
+      if (xdt == LM_F32 && (b.simt_tile[ph] = simt_tile((int64_t)lists[ph].size(), sm_count())) != bm) {
+        lists[ph].clear();
+        build_ns_tiles(groups, g0, b.ng, ph, b.simt_tile[ph], b.simt_tile[ph], lists[ph]);
+      }
+    }
     int nparts = 0;
     if (xdt == LM_BF16) {
       // three-piece mode: no fp32 accumulation over more than kGramCapF32TC K blocks
       split_gram_tiles(groups, g0, b.ng, lists[NS_GRAM], kTcBM, kTcBK, tc_max_pairs(), targets, nparts,
                        pieces == 3 ? kGramCapF32TC : 0);
     } else {
-      int dev = 0, sms = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      split_gram_tiles(groups, g0, b.ng, lists[NS_GRAM], kSimtBM, 16, 2 * std::max(sms, 1), targets, nparts);
+      for (int ph = 0; ph < 3; ++ph) {
+        const int parts = split_simt_tiles(groups, g0, ph, b.simt_tile[ph], lists[ph]);
+        L.simt_parts = std::max(L.simt_parts, parts);
+        split_floats = std::max(split_floats, (size_t)parts * b.simt_tile[ph] * b.simt_tile[ph]);
+      }
     }
     b.nsplit = (int)targets.size();
-    max_split = std::max(max_split, nparts);
+    split_floats = std::max(split_floats, (size_t)nparts * kTcBM * b.bn);
     L.ntargets += b.nsplit;
     std::vector<uint16_t> pt((size_t)nparts);
     for (size_t k = 0; k < targets.size(); ++k)
@@ -676,12 +747,12 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
   }
   L.off_groups = ar.add(groups.size() * sizeof(NsGroup));
   L.nmat = nmat;
+  L.ntargets = std::max(L.ntargets, L.simt_parts);
   L.off_clear = ar.add(std::max<size_t>(ns_clear_bytes(nmat, L.ntargets), 1));
-  const size_t tile_floats = (xdt == LM_BF16) ? (size_t)kTcBM * kTcBN : (size_t)kSimtBM * kSimtBN;
-  L.off_split_ws = buf.add((size_t)max_split * tile_floats * sizeof(float));
+  L.off_split_ws = buf.add(split_floats * sizeof(float));
 }
 
-// base: start of the tables (image host_img), bbase: start of the buffers.
+// base: start of the tables (their image is host_img), bbase: start of the buffers.
 static void bind_ns(NsEngine& E, char* base, char* bbase, const NsLayout& L, std::vector<char>& host_img) {
   for (size_t gi = 0; gi < E.groups.size(); ++gi) {
     E.groups[gi].X[0] = bbase + L.off_x0[gi];
@@ -716,23 +787,19 @@ static void bind_ns(NsEngine& E, char* base, char* bbase, const NsLayout& L, std
              L.part_target[bi].size() * sizeof(uint16_t));
     if (L.off_counts[bi] != 0) E.batches[bi].counts = reinterpret_cast<int*>(base + L.off_counts[bi]);
     std::vector<NsSplitTarget> st(tg.size());
-    const bool tc = E.xdt == LM_BF16;
-    const size_t es = tc ? 2 : 4;                 // A: bf16 (tensor cores) or fp32
-    const int tile = tc ? kTcBM : kSimtBM, tile_n = tc ? E.batches[bi].bn : kSimtBN;
+    const int tile = kTcBM, tile_n = E.batches[bi].bn;   // (tensor-core path)
     for (size_t k = 0; k < tg.size(); ++k) {
       const NsGroup& g = E.groups[E.batches[bi].g0 + tg[k][0]];
-      char* a = static_cast<char*>(g.A) + (size_t)tg[k][1] * g.s_pad * g.s_pad * es;
+      char* a = static_cast<char*>(g.A) + (size_t)tg[k][1] * g.s_pad * g.s_pad * 2;
       const int tm = tg[k][2], tn = tg[k][3];
-      st[k].a_tile = a + ((size_t)tm * tile * g.s_pad + (size_t)tn * tile_n) * es;
-      st[k].a_mirror = a + ((size_t)tn * tile_n * g.s_pad + (size_t)tm * tile) * es;
+      st[k].a_tile = a + ((size_t)tm * tile * g.s_pad + (size_t)tn * tile_n) * 2;
       st[k].ld = g.s_pad;
       st[k].nr = std::min(tile, g.s_pad - tm * tile);
       st[k].nc = std::min(tile_n, g.s_pad - tn * tile_n);
       st[k].first = tg[k][4];
       st[k].nparts = tg[k][5];
-      st[k].diag = tm == tn ? 1 : 0;
       st[k].mat = g.first_mat + tg[k][1];
-      st[k].plane = (tc && E.pieces == 3) ? (int64_t)g.count * g.s_pad * g.s_pad : 0;
+      st[k].plane = E.pieces == 3 ? (int64_t)g.count * g.s_pad * g.s_pad : 0;
     }
     E.batches[bi].split_targets = reinterpret_cast<NsSplitTarget*>(base + L.off_split_targets[bi]);
     if (!st.empty()) memcpy(host_img.data() + L.off_split_targets[bi], st.data(), st.size() * sizeof(NsSplitTarget));
@@ -810,6 +877,25 @@ static cudaError_t timed(Profiler* P, int fam, cudaStream_t st, F&& f) {
   return e;
 }
 
+// Where full-fp32 Newton-Schulz (LM_F32) runs on the tensor cores as three bf16
+// pieces with the main products summed in registers (NsChain::promote): for
+// sets all of whose matrices are wide enough that this is closer to the fp64
+// iteration than fp32 FMAs are.  Measured over 8 to 20000 rows and columns, four
+// kinds of input, each against fp64: from 333 up it is 0.15 to 0.8 times as
+// far with the quintic and the degree-5 minimax table, at 256 0.26 to 0.63
+// with the quintic but up to 1.2 with the table (whose first |a| is 8.5);
+// narrower matrices go either way (130 x 200: 0.37 to 6).  An msign of 1024 x
+// 1024 takes 516 us there against 1026 us.
+static bool f32_on_tensor_cores(const std::vector<std::pair<int64_t, int64_t>>& shapes, const std::vector<NsCoeffs>& co) {
+  int64_t least = 320;
+  bool small_a = true;
+  for (const NsCoeffs& c : co) small_a = small_a && std::fabs(c.a) < 4.f;
+  if (small_a) least = 256;
+  for (const auto& x : shapes)
+    if (std::min(x.first, x.second) < least) return false;
+  return !shapes.empty() && !co.empty();
+}
+
 // Per-iteration coefficients: (a_k, b_k, c_k) from a 3 * steps table, or the
 // constant (a, b, c) when the table is NULL; eps goes with every iteration.
 static std::vector<NsCoeffs> ns_schedule(int steps, const double* table, double a, double b, double c,
@@ -865,6 +951,7 @@ static lm_status run_ns(const NsEngine& E, int steps, const NsCoeffs* coeffs, un
       c.co = coeffs;
       c.fold = E.fold;
       c.pieces = E.pieces;
+      c.promote = E.promote;
       c.bn = b.bn;
       c.final_f32 = true;
       c.fuse = fuse;
@@ -900,11 +987,8 @@ static lm_status run_ns(const NsEngine& E, int steps, const NsCoeffs* coeffs, un
               r = launch_ns_split_finish(b.split_targets, b.nsplit, E.d_split_ws, flags, st);
             return r;
           }
-          cudaError_t r = launch_ns_simt((NsPhase)ph, it, b.ng, E.d_groups + b.g0, b.tiles[ph], b.ntiles[ph],
-                                         E.d_norm2, co, st, active, E.d_split_ws, flags);
-          if (r == cudaSuccess && split)
-            r = launch_ns_split_finish_f32(b.split_targets, b.nsplit, E.d_split_ws, flags, st);
-          return r;
+          return launch_ns_simt((NsPhase)ph, it, b.simt_tile[ph], E.d_groups + b.g0, b.tiles[ph], b.ntiles[ph],
+                                E.d_norm2, co, st, active, E.d_split_ws, b.parts_done, flags);
         });
         if (e != cudaSuccess) return cuda_fail(e, "Newton-Schulz launch");
       }
@@ -1098,8 +1182,10 @@ lm_status lm_shard_owners(const lm_tensor* params, int n, int world, int* owner)
   return LM_OK;
 }
 
-lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* cuda_stream,
-                    lm_state** out) {
+}  // extern "C"
+
+static lm_status create_state(const lm_tensor* params, int n, const lm_config* cfg, bool f32_tc, bool* used_tc,
+                              void* cuda_stream, lm_state** out) {
   if (out == nullptr) return fail(LM_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   if (params == nullptr || cfg == nullptr) return fail(LM_ERR_INVALID_ARG, "params/cfg is NULL");
@@ -1123,6 +1209,17 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   s->params.assign(params, params + n);
   s->ns.xdt = (cfg->ns_precision == LM_F32 || env_is("LM_NS_FORCE_FP32", "1")) ? LM_F32 : LM_BF16;
   s->ns.pieces = (s->ns.xdt == LM_BF16 && cfg->ns_precision == LM_NS_F32_TC) ? 3 : 1;
+  if (s->ns.xdt == LM_F32 && f32_tc) {
+    std::vector<std::pair<int64_t, int64_t>> shapes;   // every rank of a sharded set takes the same path
+    for (int i = 0; i < n; ++i)
+      if (is_matrix(params[i])) shapes.push_back({params[i].rows, params[i].cols});
+    if (f32_on_tensor_cores(shapes, s->ns_co)) {
+      s->ns.xdt = LM_BF16;
+      s->ns.pieces = 3;
+      s->ns.promote = true;
+      *used_tc = true;
+    }
+  }
   s->debug = env_is("LM_DEBUG", "1");
   if (env_is("LM_NVTX", "1")) g_nvtx.store(true);
 
@@ -1350,13 +1447,13 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   std::vector<size_t> guard_offs;
   if (s->debug)
     off_guard_list = ar.add((ar.guards.size() + buf.guards.size() + 1) * sizeof(size_t));
-  const size_t off_buf = align_up(ar.total, 256);   // the buffers follow the tables
-  const size_t total = off_buf + buf.total;
+  const size_t off_tab = align_up(buf.total, 256);   // the tables follow the buffers
+  const size_t total = off_tab + ar.total;
   if (s->debug) {
-    guard_offs = ar.guards;   // now including the list's own guard
-    for (size_t g : buf.guards) guard_offs.push_back(off_buf + g);
+    guard_offs = buf.guards;
+    for (size_t g : ar.guards) guard_offs.push_back(off_tab + g);   // now including the list's own guard
   }
-  if (env_is("LM_FAULT", "oom")) {
+  if (env_is("LM_FAULT", "oom") || (s->ns.promote && env_is("LM_FAULT", "oom_f32tc"))) {
     delete s;
     return fail(LM_ERR_OOM, "injected allocation failure (LM_FAULT=oom)");
   }
@@ -1370,11 +1467,11 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   if (s->debug) {
     for (size_t g : ar.guards) memset(img.data() + g, kGuardByte, kGuardBytes);
     memcpy(img.data() + off_guard_list, guard_offs.data(), guard_offs.size() * sizeof(size_t));
-    s->d_guard_offs = reinterpret_cast<size_t*>(s->base + off_guard_list);
+    s->d_guard_offs = reinterpret_cast<size_t*>(s->base + off_tab + off_guard_list);
     s->n_guards = (int)guard_offs.size();
   }
-  char* base = s->base;
-  char* bbase = s->base + off_buf;
+  char* base = s->base + off_tab;
+  char* bbase = s->base;
   s->mom = reinterpret_cast<float*>(bbase + off_mom);
   s->d_grads = reinterpret_cast<const void**>(base + off_grads);
   s->d_flags = reinterpret_cast<unsigned*>(base + off_flags);
@@ -1528,6 +1625,19 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* 
   s->last_stream = stream;
   *out = s;
   return LM_OK;
+}
+
+extern "C" {
+
+lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg, void* cuda_stream, lm_state** out) {
+  bool used_tc = false;
+  lm_status st = create_state(params, n, cfg, true, &used_tc, cuda_stream, out);
+  // no room for the three-piece workspace: the CUDA-core path needs half of it
+  if (st == LM_ERR_OOM && used_tc) {
+    cudaGetLastError();
+    st = create_state(params, n, cfg, false, &used_tc, cuda_stream, out);
+  }
+  return st;
 }
 
 static lm_status upload_grads(lm_state* s, const lm_tensor* grads, cudaStream_t st) {
@@ -1952,8 +2062,8 @@ void lm_destroy(lm_state* s) {
 // The msign entry points: norm kernel, NS iterations with per-iteration
 // coefficients co[0 .. steps-1], output kernel; arguments already checked
 // except the tensors and the size limits.
-static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, const std::vector<NsCoeffs>& co,
-                            double eps, int precision, void* cuda_stream) {
+static lm_status msign_run(const lm_tensor* in, lm_tensor* out, int steps, const std::vector<NsCoeffs>& co,
+                           double eps, int precision, bool f32_tc, void* cuda_stream) {
   lm_status st;
   if ((st = check_tensor(in, "in", 0)) != LM_OK) return st;
   if ((st = check_tensor(out, "out", 0)) != LM_OK) return st;
@@ -1970,6 +2080,11 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   NsEngine E;
   E.xdt = precision == LM_F32 ? LM_F32 : LM_BF16;
   E.pieces = precision == LM_NS_F32_TC ? 3 : 1;
+  if (f32_tc) {
+    E.xdt = LM_BF16;
+    E.pieces = 3;
+    E.promote = true;
+  }
   const lm_dtype xio = E.pieces == 3 ? LM_F32 : E.xdt;   // X_0 / X_K buffer dtype
   std::vector<std::vector<int>> members;
   plan_groups({{in->rows, in->cols}}, E.xdt, E.groups, members);
@@ -1989,12 +2104,13 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   const size_t off_et = ar.add(et.size() * sizeof(ElemChunk));
   const size_t off_flags = ar.add(sizeof(unsigned));
 
-  const size_t off_buf = align_up(ar.total, 256);
-  char* base = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), off_buf + buf.total, stream);
+  const size_t off_tab = align_up(buf.total, 256);
+  char* mem = nullptr;
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&mem), off_tab + ar.total, stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(msign workspace)");
+  char* base = mem + off_tab;
   std::vector<char> img(ar.total, 0);
-  bind_ns(E, base, base + off_buf, L, img);
+  bind_ns(E, base, mem, L, img);
   const NsGroup& g = E.groups[0];
   d.w = in->data;
   d.m = nullptr;
@@ -2010,7 +2126,7 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   memcpy(img.data() + off_mat, &d, sizeof(d));
   memcpy(img.data() + off_et, et.data(), et.size() * sizeof(ElemChunk));
   auto cleanup = [&](lm_status r) {
-    cudaFreeAsync(base, stream);
+    cudaFreeAsync(mem, stream);
     return r;
   };
   e = cudaMemcpyAsync(base, img.data(), ar.total, cudaMemcpyHostToDevice, stream);
@@ -2042,11 +2158,23 @@ static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, cons
   unsigned hflags = 0;
   e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  cudaFreeAsync(base, stream);
+  cudaFreeAsync(mem, stream);
   if (e != cudaSuccess) return cuda_fail(e, "msign status read");
   if (hflags & LM_FLAG_TIMEOUT)
     return fail(LM_ERR_TIMEOUT, "a bounded device wait gave up; out was not written (LM_FLAG_TIMEOUT)");
   return LM_OK;
+}
+
+static lm_status msign_impl(const lm_tensor* in, lm_tensor* out, int steps, const std::vector<NsCoeffs>& co,
+                            double eps, int precision, void* cuda_stream) {
+  const bool f32_tc = precision == LM_F32 && f32_on_tensor_cores({{in->rows, in->cols}}, co);
+  lm_status st = msign_run(in, out, steps, co, eps, precision, f32_tc, cuda_stream);
+  // no room for the three-piece workspace: the CUDA-core path needs half of it
+  if (st == LM_ERR_OOM && f32_tc) {
+    cudaGetLastError();
+    st = msign_run(in, out, steps, co, eps, precision, false, cuda_stream);
+  }
+  return st;
 }
 
 extern "C" {

@@ -160,27 +160,24 @@ struct NsGroup {
 // Tile work item: group, matrix-in-group, tile row, tile col.
 struct alignas(16) NsTile {
   uint16_t group, mat, tm, tn;
-  // Split-K (Gram phase only): K blocks [kb0, kb1) of the tile, kb1 == 0 for
-  // all of them; slot != 0: the partial product is written in fp32 to
-  // workspace tile slot - 1 instead of A (NsSplitTarget sums the parts).
+  // Split-K (the Gram phase; any phase of the fp32 path): K blocks [kb0, kb1)
+  // of the tile, kb1 == 0 for all of them; slot != 0: the partial product is
+  // written in fp32 to workspace tile slot - 1, and the parts are summed.
   uint16_t kb0, kb1, slot;
   // 256-column output blocks of the tile, starting at block tn: 2 only in
-  // the wide-tile kernel's launches (0 and 1 both mean one block).
+  // the wide-tile kernel's launches (0 and 1 both mean one block); the fp32
+  // path's split tiles: part index << 8 | parts.
   uint16_t nh;
 };
-// A split Gram tile (tile edge `tile`: 256 tensor-core, 128 fp32 path): the
+// A split Gram tile of the tensor-core path (256 rows, 256 or 128 columns): the
 // parts in workspace tiles first .. first + nparts - 1 are summed in that
 // order (so the result does not depend on timing) and written to A at
-// (tm * tile + r, tn * tile + c) for r < nr, c < nc; the fp32 path, which keeps
-// A whole, also writes the mirror (tn * tile + c, tm * tile + r), and on a
-// diagonal tile only c >= r.
+// (row0 + r, col0 + c) for r < nr, c < nc.
 struct NsSplitTarget {
-  void* a_tile;           // element (tm * tile, tn * tile) of the matrix's A
-  void* a_mirror;         // element (tn * tile, tm * tile) (fp32 path)
+  void* a_tile;           // element (row0, col0) of the matrix's A
   int32_t ld;             // s_pad
   int32_t nr, nc;         // rows / columns of the tile inside the padded matrix
   int32_t first, nparts;
-  int32_t diag;
   int32_t mat;            // matrix id
   int64_t plane;          // three-piece A: elements between its bf16 planes (0: one bf16 plane)
 };
@@ -277,6 +274,7 @@ struct NsChain {
   const NsCoeffs* co;           // host, one per iteration
   bool fold;
   int pieces;                   // 1: bf16 operands; 3: fp32 as three bf16 pieces
+  bool promote;                 // three pieces: main products summed in registers per K block (the full-fp32 mode)
   int bn;                       // columns of a tile: 256, or 128 (always with three pieces; not with a parameter
                                 // write whose iteration does not fold a)
   bool final_f32;               // three pieces: the last APPLY writes fp32 X to NsGroup::Xf
@@ -309,16 +307,21 @@ cudaError_t launch_split3(const float* src, void* dst, size_t n, const unsigned*
 cudaError_t launch_ns_split_finish(const NsSplitTarget* targets, int n, const float* ws, const unsigned* flags,
                                    cudaStream_t st);
 
-// fp32 CUDA-core path.
-constexpr int kSimtBM = 128, kSimtBN = 128;
+// fp32 CUDA-core path: square tiles of 128 or 64.
+constexpr int kSimtBM = 128;   // s and l are padded to it
 int simt_pad(int x);
-cudaError_t launch_ns_simt(NsPhase ph, int iter, int ngroups, const NsGroup* dgroups,
-                           const NsTile* tiles, int ntiles, const double* norm2, NsCoeffs co,
-                           cudaStream_t st, const unsigned char* active = nullptr, float* split_ws = nullptr,
-                           const unsigned* flags = nullptr);
-// fp32 path: A tiles (and mirrors) from the fp32 parts of split Gram tiles.
-cudaError_t launch_ns_split_finish_f32(const NsSplitTarget* targets, int n, const float* ws, const unsigned* flags,
-                                       cudaStream_t st);
+int simt_blocks(int tile, int sms);   // resident blocks of the kernel for a tile
+// Tile of a phase with `tiles128` tiles of 128: 64 where those would leave more
+// than a fifth of the last round's blocks without work (or a single round
+// short), 128 otherwise.
+int simt_tile(int64_t tiles128, int sms);
+constexpr int simt_slice(int tile) { return tile == 128 ? 16 : 32; }   // K slice (NsTile::kb0, kb1)
+// Split tiles (any phase): NsTile::slot = part + 1, nh = index << 8 | parts;
+// parts_done: one counter per part (the first of a tile's parts is used),
+// zero before the first launch, left at zero.
+cudaError_t launch_ns_simt(NsPhase ph, int iter, int tile, const NsGroup* dgroups, const NsTile* tiles, int ntiles,
+                           const double* norm2, NsCoeffs co, cudaStream_t st, const unsigned char* active,
+                           float* split_ws, uint32_t* parts_done, const unsigned* flags);
 // active (both NS paths): NULL, or active[first_mat + mat] != 0 for the
 // matrices whose tiles run; tiles of the others are skipped by every role.
 

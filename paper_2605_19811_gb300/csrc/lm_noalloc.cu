@@ -102,7 +102,7 @@ struct BuildArgs {
   int n_chunks;
   int64_t chunk;
   NsTile* d_tiles[3];
-  int bm, bn;
+  int bm[3], bn[3];
   double* d_norm2;
   uint32_t* d_done;
   unsigned* d_flags;
@@ -128,12 +128,12 @@ __global__ void build_tables_kernel(BuildArgs a) {
     const NsGroup& g = a.group;
     const int nrow = (ph == NS_APPLY && g.tall) ? g.l_pad : g.s_pad;
     const int ncol = ph == NS_APPLY ? (g.tall ? g.s_pad : g.l_pad) : g.s_pad;
-    const int tms = (nrow + a.bm - 1) / a.bm;
-    const int tns = (ncol + a.bn - 1) / a.bn;
+    const int tms = (nrow + a.bm[ph] - 1) / a.bm[ph];
+    const int tns = (ncol + a.bn[ph] - 1) / a.bn[ph];
     int k = 0;
     for (int tm = 0; tm < tms; ++tm)
       for (int tn = 0; tn < tns; ++tn) {
-        if (ph != NS_APPLY && (int64_t)(tn + 1) * a.bn <= (int64_t)tm * a.bm) continue;
+        if (ph != NS_APPLY && (int64_t)(tn + 1) * a.bn[ph] <= (int64_t)tm * a.bm[ph]) continue;
         a.d_tiles[ph][k++] = NsTile{0, 0, (uint16_t)tm, (uint16_t)tn};
       }
   }
@@ -188,14 +188,26 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   const int s = (int)std::min(in->rows, in->cols), l = (int)std::max(in->rows, in->cols);
   const int s_pad = xdt == LM_BF16 ? tc_pad_s(s) : simt_pad(s);
   const int l_pad = xdt == LM_BF16 ? tc_pad_l(l) : simt_pad(l);
-  const int bm = xdt == LM_BF16 ? kTcBM : kSimtBM;
-  const int bn = xdt == LM_BF16 ? tc_tile_cols(phase_tiles(NS_APPLY, s_pad, l_pad, in->rows > in->cols, bm, kTcBN), 1)
-                                : kSimtBN;
   const size_t es = xdt == LM_BF16 ? 2 : 4;
   const int tall = in->rows > in->cols ? 1 : 0;
   const int64_t numel = in->rows * in->cols;
-  int ntiles[3];
-  for (int ph = 0; ph < 3; ++ph) ntiles[ph] = phase_tiles(ph, s_pad, l_pad, tall, bm, bn);
+  const size_t xbytes = (size_t)s_pad * l_pad * es, abytes = (size_t)s_pad * s_pad * es;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // smaller tiles and chunks need longer tables (well below 1 MiB): only
+  // where the area has that to spare, so that they never cost a matrix its room
+  const bool roomy = 2 * (xbytes + abytes) + ((size_t)1 << 20) <= kNoAllocScratchBytes;
+  int tile_rows[3], tile_cols[3], ntiles[3];
+  for (int ph = 0; ph < 3; ++ph) {
+    if (xdt == LM_BF16) {
+      tile_rows[ph] = kTcBM;
+      tile_cols[ph] = roomy ? tc_tile_cols(phase_tiles(NS_APPLY, s_pad, l_pad, tall, kTcBM, kTcBN), 1) : kTcBN;
+    } else {
+      const int n128 = phase_tiles(ph, s_pad, l_pad, tall, kSimtBM, kSimtBM);
+      tile_rows[ph] = tile_cols[ph] = roomy ? simt_tile(n128, sms) : kSimtBM;
+    }
+    ntiles[ph] = phase_tiles(ph, s_pad, l_pad, tall, tile_rows[ph], tile_cols[ph]);
+  }
 
   size_t off = 0;
   const size_t off_flags = off;   off = align256(off + sizeof(unsigned));
@@ -207,16 +219,11 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
     off_tiles[ph] = off;
     off = align256(off + (size_t)ntiles[ph] * sizeof(NsTile));
   }
-  const size_t xbytes = (size_t)s_pad * l_pad * es, abytes = (size_t)s_pad * s_pad * es;
   const size_t off_x0 = off;  off = align256(off + xbytes);
   const size_t off_x1 = off;  off = align256(off + xbytes);
   const size_t off_a = off;   off = align256(off + abytes);
   const size_t off_b = off;   off = align256(off + abytes);
-  // the element chunks come last: short ones where their table still fits
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t chunk = elem_chunk(numel, sms);
-  if (off + (size_t)((numel + chunk - 1) / chunk) * sizeof(ElemChunk) > kNoAllocScratchBytes) chunk = kElemChunk;
+  const int64_t chunk = roomy ? elem_chunk(numel, sms) : kElemChunk;
   const int n_et = (int)((numel + chunk - 1) / chunk);
   const size_t off_et = off;  off = align256(off + (size_t)n_et * sizeof(ElemChunk));
   if (off > kNoAllocScratchBytes) {
@@ -272,15 +279,17 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   ba.n_chunks = n_et;
   ba.chunk = chunk;
   for (int ph = 0; ph < 3; ++ph) ba.d_tiles[ph] = reinterpret_cast<NsTile*>(base + off_tiles[ph]);
-  ba.bm = bm;
-  ba.bn = bn;
+  for (int ph = 0; ph < 3; ++ph) {
+    ba.bm[ph] = tile_rows[ph];
+    ba.bn[ph] = tile_cols[ph];
+  }
   ba.d_norm2 = d.norm2;
   ba.d_done = reinterpret_cast<uint32_t*>(d.norm2 + 1);
   ba.d_flags = reinterpret_cast<unsigned*>(base + off_flags);
 
   TcGroupMaps maps;
   if (xdt == LM_BF16) {
-    e = tc_encode_group_maps(g, &maps, 1, bn, false);
+    e = tc_encode_group_maps(g, &maps, 1, tile_cols[NS_GRAM], false);
     if (e != cudaSuccess) return set_error(LM_ERR_CUDA, "cuTensorMapEncodeTiled failed");
   }
 
@@ -318,7 +327,7 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
     ch.co = cos.data();
     ch.fold = !(fold_env != nullptr && std::strcmp(fold_env, "0") == 0);
     ch.pieces = 1;
-    ch.bn = bn;
+    ch.bn = tile_cols[NS_GRAM];
     ch.flags = ba.d_flags;
     ch.wait_ns = env_wait_limit_ns();
     e = launch_ns_chain(ch, 0, 3 * steps, stream);
@@ -326,8 +335,8 @@ extern "C" lm_status lm_msign_ns_noalloc(const lm_tensor* in, lm_tensor* out, in
   }
   for (int it = 0; it < steps && xdt == LM_F32; ++it)
     for (int ph = 0; ph < 3; ++ph) {
-      e = launch_ns_simt((NsPhase)ph, it, 1, ba.d_group, ba.d_tiles[ph], ntiles[ph], d.norm2, co, stream, nullptr,
-                         nullptr, ba.d_flags);
+      e = launch_ns_simt((NsPhase)ph, it, tile_rows[ph], ba.d_group, ba.d_tiles[ph], ntiles[ph], d.norm2, co, stream,
+                         nullptr, nullptr, nullptr, ba.d_flags);
       if (e != cudaSuccess) return set_error(LM_ERR_CUDA, cudaGetErrorString(e));
     }
   e = launch_finalize(xdt, out->dtype, ba.d_mat, ba.d_chunks, n_et, mk, 1, ba.d_flags, stream);

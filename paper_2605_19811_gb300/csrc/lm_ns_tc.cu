@@ -88,9 +88,8 @@ constexpr int kTmemCols = 512;
 //   kP = 1 (bf16 operands), 256 columns: a 5-stage ring of 32 KB per CTA and
 //     a 64 KB aux/staging buffer; 128 columns: 8 stages of 24 KB and 32 KB.
 //   kP = 3 (fp32 operands held as three bf16 pieces hi + mid + lo, exact), 128
-//     columns: a 3-stage ring of 72 KB per CTA and a 32 x 17 fp32 transpose
-//     tile per epilogue warp (that epilogue reads its aux values and writes
-//     its results through global memory).
+//     columns: a 3-stage ring of 72 KB per CTA (the epilogue reads its aux
+//     values and writes its results through global memory).
 template <int kP, int kBN>
 struct TcLayout {
   static constexpr int kBBytes = kBN / 2 * BK * 2;        // a CTA's half of a B operand block
@@ -98,7 +97,7 @@ struct TcLayout {
   static constexpr int kStageBytes = kP * (kABytes + kBBytes);
   static constexpr int kBoxes = kBN / 64;
   static constexpr size_t kAuxOffset = (size_t)kStages * kStageBytes;
-  static constexpr size_t kBarOffset = kAuxOffset + (kP == 1 ? kBoxes * kAuxBoxBytes : 4 * 32 * 17 * 4);
+  static constexpr size_t kBarOffset = kAuxOffset + (kP == 1 ? kBoxes * kAuxBoxBytes : 0);
   static constexpr size_t kSmemBytes = 1024 /*align slack*/ + kBarOffset + 512;
   static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 };
@@ -221,19 +220,32 @@ __device__ __forceinline__ bool produce_range(ProducerRing<TcLayout<kP, kBN>::kS
 // kP = 3: with A = A0 + A1 + A2 and B = B0 + B1 + B2 (each piece 2^-8 of the
 // previous in magnitude) the six products of order up to 2^-16 are summed,
 // A0B0 + A0B1 + A1B0 + A0B2 + A2B0 + A1B1; the dropped ones are of order 2^-24.
-// A0B0 goes into the accumulator d_tmem and the five smaller products into
-// d_cross; the epilogue adds the two in fp32.  The tensor cores' fp32
-// accumulation loses about one unit of the last place of the accumulator per
-// MMA, in the same direction (measured: the error grows with the number of
-// MMAs summed, 2.2e-5 relative for a 1280-deep product with all six in one
-// accumulator), so the large accumulator takes a sixth of the additions and
-// the errors of the other are 2^-8 smaller.
-template <bool AMN, bool BMN, int kP, int kBN>
+// The tensor cores' fp32 accumulation loses about one unit of the last place of
+// the accumulator per MMA, always in the same direction (2.2e-5 relative for a
+// 1280-deep product with all six in one accumulator), so A0B0 has one of its
+// own and the five smaller products, 2^-8 of it, share another (4.4e-6).
+// kPromo (the full-fp32 mode): A0B0 is accumulated for one K block only (four
+// MMAs), in one of two accumulators by turns, and the epilogue warps add each
+// block's sum to theirs in fp32 registers, rounded to nearest, while the next
+// block runs.  Five iterations of the quintic are then 0.2 to 0.63 times as far
+// from fp64 as with fp32 FMAs on the CUDA cores (256 to 5120 wide: 4.5e-7 to
+// 1.4e-6 against 1.6e-6 to 3.3e-6; dropping no product at all, eight of them,
+// changes nothing).  Its cost: the warps that hold the sums cannot go on adding
+// while they write a tile out, so the MMAs of the next tile wait (4-layer d =
+// 1280 set: 10.7 ms per Muon step against 7.6 without).
+// Main products: per K block n, accumulator n & 1; mfull: the block's four MMAs
+// are done (both CTAs), mempty: every epilogue warp has read it.
+struct MainRing {
+  uint32_t n;          // K blocks issued
+  uint32_t tmem;       // columns of accumulator 0
+  uint64_t* mfull;
+  uint64_t* mempty;
+};
+template <bool AMN, bool BMN, int kP, int kBN, bool kPromo>
 __device__ __forceinline__ bool mma_range(int& stage, uint32_t& ph, uint8_t* smem, uint64_t* full,
                                           uint64_t* empty, volatile int* abort_flag, uint64_t wait_ns, int kb0,
-                                          int kb1, uint32_t d_tmem, uint32_t d_cross, int kb_first, bool same) {
+                                          int kb1, uint32_t d_tmem, MainRing& mr, int kb_first, bool same) {
   using L = TcLayout<kP, kBN>;
-  constexpr int kProducts = kP == 1 ? 1 : 6;
   constexpr int qa[6] = {0, 0, 1, 0, 2, 1};
   constexpr int qb[6] = {0, 1, 0, 2, 0, 1};
   const uint32_t idesc = make_idesc(BM, kBN, AMN, BMN);
@@ -247,15 +259,32 @@ __device__ __forceinline__ bool mma_range(int& stage, uint32_t& ph, uint8_t* sme
     // shared-memory window is below 2^18 bytes)
     const uint64_t a0 = AMN ? sw128_desc(sa, 64 * BK * 2, 1024) : sw128_desc(sa, 16, 1024);
     const uint64_t b0 = BMN ? sw128_desc(sb, 64 * BK * 2, 1024) : sw128_desc(sb, 16, 1024);
+    auto step = [&](int m, int kk, uint32_t d, bool first) {
+      const uint64_t adesc = a0 + (uint64_t)((qa[m] * kABytes + kk * (AMN ? 2048 : 32)) >> 4);
+      const uint64_t bdesc = b0 + (uint64_t)((qb[m] * L::kBBytes + kk * (BMN ? 2048 : 32)) >> 4);
+      umma_bf16(d, adesc, bdesc, idesc, first ? 0u : 1u);
+    };
+    if constexpr (kP == 1) {
 #pragma unroll
-    for (int kk = 0; kk < BK / 16; ++kk) {
+      for (int kk = 0; kk < BK / 16; ++kk) step(0, kk, d_tmem, kb == kb_first && kk == 0);
+    } else if constexpr (!kPromo) {
 #pragma unroll
-      for (int m = 0; m < kProducts; ++m) {
-        const uint64_t adesc = a0 + (uint64_t)((qa[m] * kABytes + kk * (AMN ? 2048 : 32)) >> 4);
-        const uint64_t bdesc = b0 + (uint64_t)((qb[m] * L::kBBytes + kk * (BMN ? 2048 : 32)) >> 4);
-        const bool first = kb == kb_first && kk == 0 && m <= 1;   // first product into each accumulator
-        umma_bf16(m == 0 ? d_tmem : d_cross, adesc, bdesc, idesc, first ? 0u : 1u);
-      }
+      for (int kk = 0; kk < BK / 16; ++kk)
+#pragma unroll
+        for (int m = 0; m < 6; ++m)
+          step(m, kk, m == 0 ? d_tmem : d_tmem + (uint32_t)kBN, kb == kb_first && kk == 0 && m <= 1);
+    } else {
+      const uint32_t mb = mr.n & 1u;
+      if (!mbar_wait(&mr.mempty[mb], ((mr.n >> 1) & 1u) ^ 1u, abort_flag, wait_ns)) return false;
+      tc_fence_after();
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk) step(0, kk, mr.tmem + mb * (uint32_t)kBN, kk == 0);
+      umma_commit_pair(&mr.mfull[mb]);
+      ++mr.n;
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk)
+#pragma unroll
+        for (int m = 1; m < 6; ++m) step(m, kk, d_tmem, kb == kb_first && kk == 0 && m == 1);
     }
     umma_commit_pair(&empty[stage]);
     if (++stage == L::kStages) {
@@ -276,77 +305,77 @@ __device__ __forceinline__ void split3(float v, float& h, float& m, float& l) {
 }
 // Epilogue of one 32 x 16 chunk (rows r0 .. r0 + 31, one per lane; columns
 // j0 ..) with three-piece operands; aux values and results go through global
-// memory, coalesced through the warp's transpose tile stg: lane l reads and
-// writes 16 bytes of row l / 2 + 16 k (k = 0, 1), so a warp access covers 16
-// rows x 32 bytes of one plane.
+// memory in whole 32-byte sectors: lanes 2m and 2m + 1 access the two halves of
+// row 2m, then of row 2m + 1, and exchange the halves that are not theirs.
 //   kacc: APPLY's factor on the accumulator (1, or b where B = b A was not
 //   formed).
 //   aux: the A (POLY) or X (APPLY) element, hi + mid + lo; out: the result's
 //   pieces, or fp32 in out_f32 (last APPLY).  base: element (r0, j0) of the
 //   matrix in plane 0; ld: row length; plane: elements per piece.
 template <typename Co>
-__device__ __forceinline__ void piece_chunk(const uint32_t (&r)[16], int phase, const Co& co, float nscale,
+__device__ __forceinline__ void piece_chunk(const float (&acc)[16], int phase, const Co& co, float nscale,
                                             float kacc,
                                             const __nv_bfloat16* aux, __nv_bfloat16* out, float* out_f32,
                                             size_t plane, size_t base, size_t ld, bool row_ok, int j0, int ncols,
-                                            float (*stg)[17], int lane) {
-  const int rr = lane >> 1, c8 = (lane & 1) * 8;
+                                            int lane) {
+  const bool odd = lane & 1;
+  const size_t off0 = base + (size_t)(lane & ~1) * ld + (odd ? 8 : 0);   // this lane's half of row 2m
   float v[16];
   if (phase != NS_GRAM) {
+    float h[2][8];   // this lane's halves of rows 2m and 2m + 1
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const int row = rr + 16 * k;
-      float a8[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) a8[t] = 0.f;
+      for (int t = 0; t < 8; ++t) h[k][t] = 0.f;
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         // through L2: another SM may have written the tile in this launch
-        const uint4 a4 = __ldcg(reinterpret_cast<const uint4*>(aux + q * plane + base + (size_t)row * ld + c8));
+        const uint4 a4 = __ldcg(reinterpret_cast<const uint4*>(aux + q * plane + off0 + (size_t)k * ld));
         const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          a8[2 * e] += bf_lo(aw[e]);
-          a8[2 * e + 1] += bf_hi(aw[e]);
+          h[k][2 * e] += bf_lo(aw[e]);
+          h[k][2 * e + 1] += bf_hi(aw[e]);
         }
       }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) stg[row][c8 + t] = a8[t];
     }
-    __syncwarp();
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = stg[lane][e];
-    __syncwarp();
+    for (int t = 0; t < 8; ++t) {   // an even lane owns row 2m, an odd one row 2m + 1
+      const float got = __shfl_xor_sync(0xffffffffu, odd ? h[0][t] : h[1][t], 1);
+      v[t] = odd ? got : h[0][t];
+      v[8 + t] = odd ? h[1][t] : got;
+    }
   }
+  float o[16];
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
-    const float acc = __uint_as_float(r[e]);
-    float o;
-    if (phase == NS_GRAM) o = acc * nscale;
-    else if (phase == NS_POLY) o = poly_value(co.b, v[e], co.c, acc);
-    else o = __fmaf_rn(co.a, v[e], kacc * acc) * nscale;   // kacc = 1: exactly a v + acc, one rounding
-    stg[lane][e] = (row_ok && j0 + e < ncols) ? o : 0.f;
+    if (phase == NS_GRAM) o[e] = acc[e] * nscale;
+    else if (phase == NS_POLY) o[e] = poly_value(co.b, v[e], co.c, acc[e]);
+    else o[e] = __fmaf_rn(co.a, v[e], kacc * acc[e]) * nscale;   // kacc = 1: exactly a v + acc, one rounding
+    o[e] = (row_ok && j0 + e < ncols) ? o[e] : 0.f;
   }
-  __syncwarp();
+  float h[2][8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const float got = __shfl_xor_sync(0xffffffffu, odd ? o[t] : o[8 + t], 1);
+    h[0][t] = odd ? got : o[t];
+    h[1][t] = odd ? o[8 + t] : got;
+  }
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const int row = rr + 16 * k;
-    float o8[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) o8[t] = stg[row][c8 + t];
-    const size_t off = base + (size_t)row * ld + c8;
+    const size_t off = off0 + (size_t)k * ld;
     if (out_f32 != nullptr) {
       float4* dst = reinterpret_cast<float4*>(out_f32 + off);
-      dst[0] = make_float4(o8[0], o8[1], o8[2], o8[3]);
-      dst[1] = make_float4(o8[4], o8[5], o8[6], o8[7]);
+      dst[0] = make_float4(h[k][0], h[k][1], h[k][2], h[k][3]);
+      dst[1] = make_float4(h[k][4], h[k][5], h[k][6], h[k][7]);
       continue;
     }
     uint32_t w[3][4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       float h0, m0, l0, h1, m1, l1;
-      split3(o8[2 * e], h0, m0, l0);
-      split3(o8[2 * e + 1], h1, m1, l1);
+      split3(h[k][2 * e], h0, m0, l0);
+      split3(h[k][2 * e + 1], h1, m1, l1);
       w[0][e] = pack_bf2(h0, h1);
       w[1][e] = pack_bf2(m0, m1);
       w[2][e] = pack_bf2(l0, l1);
@@ -355,7 +384,6 @@ __device__ __forceinline__ void piece_chunk(const uint32_t (&r)[16], int phase, 
     for (int q = 0; q < 3; ++q)
       *reinterpret_cast<uint4*>(out + q * plane + off) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
   }
-  __syncwarp();   // the tile is reused by the next chunk
 }
 
 // ------------------------------- the chain ----------------------------------
@@ -540,14 +568,17 @@ __device__ __forceinline__ void finish_unit(const NsSplitTarget& T, const float*
   }
 }
 
+__device__ __forceinline__ float as_float(uint32_t v) { return __uint_as_float(v); }
+__device__ __forceinline__ float as_float(float v) { return v; }
 // 32 columns of a partial Gram product to its fp32 workspace row (zeros
 // outside the true extent), in 32-byte stores.
-__device__ __forceinline__ void split_chunk(const uint32_t (&r)[32], float* dst, float nscale, bool row_ok, int ncols) {
+template <typename V>
+__device__ __forceinline__ void split_chunk(const V (&r)[32], float* dst, float nscale, bool row_ok, int ncols) {
 #pragma unroll
   for (int e = 0; e < 32; e += 8) {
     float o[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) o[u] = (row_ok && e + u < ncols) ? __uint_as_float(r[e + u]) * nscale : 0.f;
+    for (int u = 0; u < 8; ++u) o[u] = (row_ok && e + u < ncols) ? as_float(r[e + u]) * nscale : 0.f;
     st_global_v8(dst + e, o);
   }
 }
@@ -657,7 +688,7 @@ __device__ __forceinline__ void epi_boxes(uint32_t acc, uint8_t* rowbase, int rx
 // kSplit: the Gram tiles include split-K parts (the plain instantiation keeps
 // the common path free of them).  kP: bf16 pieces per operand value (1: bf16
 // operands; 3: fp32 operands as hi + mid + lo bf16 pieces, six products).
-template <bool kSplit, int kP, int kBN>
+template <bool kSplit, int kP, int kBN, bool kPromo>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
     ns_tc_kernel(const __grid_constant__ ChainParams p) {
   using L = TcLayout<kP, kBN>;
@@ -665,7 +696,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
   // tiles in flight in TMEM: kP = 1 double-buffers two accumulators; kP = 3
   // gives one tile both (main and cross products)
   constexpr int kAccRing = kAccBufs;
-  constexpr int kAccCols = kP == 1 ? kBN : 2 * kBN;   // kP = 3: main and cross products
+  constexpr int kAccCols = kP == 3 && !kPromo ? 2 * kBN : kBN;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -678,7 +709,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
   uint64_t* done = aux_full + 1;
   uint64_t* box_full = done + 1;    // per 64-column box of auxbuf: results written, ready to store
   uint64_t* box_free = box_full + 4;   // all four stored (read by the TMA): auxbuf may be rewritten
-  ProducerLog<kStages>* log = reinterpret_cast<ProducerLog<kStages>*>(box_free + 1);
+  uint64_t* mfull = box_free + 1;      // three pieces: main-product accumulators (MainRing)
+  uint64_t* mempty = mfull + 2;
+  ProducerLog<kStages>* log = reinterpret_cast<ProducerLog<kStages>*>(mempty + 2);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(log + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* stop_word = tmem_slot + 2;
@@ -729,6 +762,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
     mbar_init(done, 1);
     for (int b = 0; b < 4; ++b) mbar_init(&box_full[b], 4);   // four warps (lane quadrants) write a box
     mbar_init(box_free, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&mfull[b], 1);
+      mbar_init(&mempty[b], 2 * nepi);
+    }
     log->n = 0;
     *abort_flag = 0;
     *aux_left = 0u;
@@ -802,6 +839,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       int ab = 0;
       uint32_t aph = 0;
       bool ok = true;
+      MainRing mr{0u, tmem_base + (uint32_t)(2 * kBN), mfull, mempty};   // kP = 3: columns behind the cross products
       for (TileStream S = tile_stream(p, pair, npairs); ok && !stopped && S.have;) {
         const NsTile t = S.t;
         const int it = S.nit, phase = S.nph;
@@ -815,23 +853,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
           break;
         }
         tc_fence_after();
-        // kP = 3: the main products in an accumulator's first kBN columns, the
-        // cross products in the second
+        // three pieces: main and cross products, or with kPromo the cross
+        // products alone
         const uint32_t d_tmem = tmem_base + (uint32_t)(ab * kAccCols);
-        const uint32_t d_cross = d_tmem + (uint32_t)kBN;
         int kb0 = P.kb_start;
 #pragma unroll 1
         for (int sg = 0; ok && sg < 3; ++sg) {
           const OpSeg S = sg == 0 ? P.s0 : (sg == 1 ? P.s1 : P.s2);
           if (S.kb_end <= kb0) continue;
           if (!S.a_mn && !S.b_mn)
-            ok = mma_range<false, false, kP, kBN>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, d_cross,
+            ok = mma_range<false, false, kP, kBN, kPromo>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, mr,
                                             P.kb_start, same);
           else if (!S.a_mn)
-            ok = mma_range<false, true, kP, kBN>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, d_cross,
+            ok = mma_range<false, true, kP, kBN, kPromo>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, mr,
                                             P.kb_start, same);
           else
-            ok = mma_range<true, true, kP, kBN>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, d_cross,
+            ok = mma_range<true, true, kP, kBN, kPromo>(stage, ph, smem, full, empty, abort_flag, wait_ns, kb0, S.kb_end, d_tmem, mr,
                                             P.kb_start, same);
           kb0 = S.kb_end;
         }
@@ -972,8 +1009,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
     const int row = q * 32 + lane;            // row of this CTA's half tile
     const uint32_t acc_empty0 = peer_addr(&accempty[0], 0);
     const uint32_t acc_empty1 = peer_addr(&accempty[kAccRing - 1], 0);
+    const uint32_t mempty0 = peer_addr(&mempty[0], 0), mempty1 = peer_addr(&mempty[1], 0);
     int ab = 0;
     uint32_t aph = 0, xph = 0, sph = 0, ntile = 0;
+    uint32_t nblk = 0;   // three pieces: K blocks whose main products this warp has added
     bool alive = !stopped;
     // Finish units of the split Gram tiles of one iteration, dealt out to all
     // eight warps of every CTA (loads in flight bound them); a warp reaches them
@@ -1023,7 +1062,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       if (kSplit) {
         while (alive && (fin_it < it || (fin_it == it && phase != NS_GRAM))) finish(nullptr, 0u);
         if (!alive) break;
-        if (phase == NS_GRAM && fin_it == it) finish(&accfull[ab], aph);
+        if (phase == NS_GRAM && fin_it == it)
+          finish(!kPromo ? &accfull[ab] : &mfull[nblk & 1u], !kPromo ? aph : (nblk >> 1) & 1u);
       }
       const NsGroup& g = p.groups[t.group];
       const ChainIter co = p.it[it];
@@ -1036,7 +1076,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       // a tile whose epilogue starts after a give-up was recorded leaves W alone
       const unsigned flags_now = global_w && lane == 0 ? *reinterpret_cast<volatile unsigned*>(p.flags) : 0u;
       const bool write_w = global_w && __shfl_sync(0xffffffffu, flags_now, 0) == 0u;
-      bool ok = mbar_wait_warp(&accfull[ab], aph, abort_flag, wait_ns);
+      bool ok = true;
+      // three pieces: half the tile's columns per warp; the main products of
+      // each K block, added in block order
+      float sum[kP == 3 ? 2 : 1][32];
+      if constexpr (kPromo) {
+        const int nk = phase != NS_GRAM ? g.s_pad / BK : (t.kb1 != 0 ? (int)t.kb1 - (int)t.kb0 : g.l_pad / BK);
+        const uint32_t main0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * kBN + half0 * (kBN / 2));
+#pragma unroll
+        for (int e = 0; e < 32; ++e) sum[0][e] = sum[1][e] = 0.f;
+#pragma unroll 1
+        for (int k = 0; ok && k < nk; ++k, ++nblk) {
+          const uint32_t mb = nblk & 1u;
+          ok = mbar_wait_warp(&mfull[mb], (nblk >> 1) & 1u, abort_flag, wait_ns);
+          if (!ok) break;
+          tc_fence_after();
+          uint32_t ra[32], rb[32];
+          tmem_ld32_async(main0 + mb * (uint32_t)kBN, ra);
+          tmem_ld32_async(main0 + mb * (uint32_t)kBN + 32u, rb);
+          tmem_ld_wait(ra);
+          tmem_ld_wait(rb);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mb == 0u ? mempty0 : mempty1);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            sum[0][e] += __uint_as_float(ra[e]);
+            sum[1][e] += __uint_as_float(rb[e]);
+          }
+        }
+      }
+      if (ok) ok = mbar_wait_warp(&accfull[ab], aph, abort_flag, wait_ns);
       if (ok && aux_phase) ok = mbar_wait_warp(aux_full, xph, abort_flag, wait_ns);
       if (!ok) {
         if (lane == 0) give_up();
@@ -1077,35 +1147,46 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         const __nv_bfloat16* aux = static_cast<const __nv_bfloat16*>(phase == NS_POLY ? g.A : g.X[cur]);
         __nv_bfloat16* out = static_cast<__nv_bfloat16*>(phase == NS_GRAM ? g.A : (phase == NS_POLY ? g.B : g.X[cur ^ 1]));
         float* out_f32 = (phase == NS_APPLY && p.final_f32 && it == p.steps - 1) ? static_cast<float*>(g.Xf) : nullptr;
-        float (*stg)[17] = reinterpret_cast<float (*)[17]>(auxbuf) + (warp - 2) * 32;
-#pragma unroll 1
-        for (int ch = 0; ch < kBN / 32; ++ch) {   // (four epilogue warps: all columns)
-          uint32_t r[32], rc[32];   // main + cross accumulators
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {   // this warp's 32-column chunks: add the cross products
+          uint32_t rc[32];
+          const uint32_t at = acc0 + (uint32_t)(half0 * (kBN / 2) + c * 32);
           __syncwarp();   // tcgen05.ld is warp-collective: reconverge first
-          tmem_ld32_async(acc0 + (uint32_t)(ch * 32), r);
-          tmem_ld32_async(acc0 + (uint32_t)(kBN + ch * 32), rc);
-          tmem_ld_wait(r);
+          if constexpr (!kPromo) {
+            uint32_t rm[32];
+            tmem_ld32_async(at, rm);
+            tmem_ld32_async(at + (uint32_t)kBN, rc);
+            tmem_ld_wait(rm);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) sum[c][e] = __uint_as_float(rm[e]);
+          } else {
+            tmem_ld32_async(at, rc);
+          }
           tmem_ld_wait(rc);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(rc[e]));
-          const int j0 = t.tn * kBN + ch * 32;
+          for (int e = 0; e < 32; ++e) sum[c][e] += __uint_as_float(rc[e]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int cc = half0 * (kBN / 2) + c * 32, j0 = t.tn * kBN + cc;
           if (!warp_in || j0 >= jmax) continue;   // beyond the padded matrix
           if (split) {
-            split_chunk(r, p.split_ws + (size_t)(t.slot - 1) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN +
-                               ch * 32, nscale, i < nrows, ncols - j0);
+            split_chunk(sum[c], p.split_ws + (size_t)(t.slot - 1) * (BM * kBN) +
+                                    (size_t)((int)rank * kHalf + row) * kBN + cc, nscale, i < nrows, ncols - j0);
             continue;
           }
           const size_t base = (size_t)t.mat * msize + (size_t)r0 * ld + j0;   // row r0 = this warp's first
-          uint32_t lo[16], hi[16];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            lo[e] = r[e];
-            hi[e] = r[16 + e];
+          for (int h = 0; h < 2; ++h) {
+            float x[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) x[e] = sum[c][16 * h + e];
+            piece_chunk(x, phase, co, nscale, kacc, aux, out, out_f32, plane, base + 16 * h, ld, i < nrows,
+                        j0 + 16 * h, ncols, lane);
           }
-          piece_chunk(lo, phase, co, nscale, kacc, aux, out, out_f32, plane, base, ld, i < nrows, j0, ncols, stg,
-                      lane);
-          piece_chunk(hi, phase, co, nscale, kacc, aux, out, out_f32, plane, base + 16, ld, i < nrows, j0 + 16, ncols,
-                      stg, lane);
         }
       } else if (split) {
         // partial Gram product of a split tile: its own fp32 workspace tile
@@ -1171,9 +1252,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         for (int b = b1; bf != nullptr && b < bn; ++b)   // nothing to store there
           if (lane == 0) mbar_arrive(&bf[b]);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
+      if constexpr (kP == 1) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
+      }
       if (++ab == kAccRing) {
         ab = 0;
         aph ^= 1u;
@@ -1449,13 +1532,13 @@ cudaError_t launch_ns_split_finish(const NsSplitTarget* targets, int n, const fl
   return cudaGetLastError();
 }
 
-template <bool kSplit, int kP, int kBN>
+template <bool kSplit, int kP, int kBN, bool kPromo = false>
 static cudaError_t set_smem_attr() {
-  return cudaFuncSetAttribute(ns_tc_kernel<kSplit, kP, kBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(ns_tc_kernel<kSplit, kP, kBN, kPromo>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)TcLayout<kP, kBN>::kSmemBytes);
 }
 
-template <bool kSplit, int kP, int kBN>
+template <bool kSplit, int kP, int kBN, bool kPromo = false>
 static cudaError_t launch_chain(const ChainParams& prm, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
@@ -1467,7 +1550,7 @@ static cudaError_t launch_chain(const ChainParams& prm, int grid, cudaStream_t s
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ns_tc_kernel<kSplit, kP, kBN>, prm);
+  return cudaLaunchKernelEx(&cfg, ns_tc_kernel<kSplit, kP, kBN, kPromo>, prm);
 }
 
 int tc_max_pairs() {
@@ -1485,7 +1568,7 @@ int tc_max_pairs() {
     cfg.blockDim = dim3(kChainThreads, 1, 1);
     cfg.dynamicSmemBytes = TcLayout<1, 256>::kSmemBytes;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, ns_tc_kernel<true, 1, 256>, &cfg) == cudaSuccess && n > 0 && n < pairs) pairs = n;
+    if (cudaOccupancyMaxActiveClusters(&n, ns_tc_kernel<true, 1, 256, false>, &cfg) == cudaSuccess && n > 0 && n < pairs) pairs = n;
   }
   cudaGetLastError();   // no device (planning on the host alone): not an error here
   if (slot >= 0) cached[slot] = pairs;
@@ -1507,6 +1590,8 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
     if (e == cudaSuccess) e = set_smem_attr<true, 1, 128>();
     if (e == cudaSuccess) e = set_smem_attr<false, 3, 128>();
     if (e == cudaSuccess) e = set_smem_attr<true, 3, 128>();
+    if (e == cudaSuccess) e = set_smem_attr<false, 3, 128, true>();
+    if (e == cudaSuccess) e = set_smem_attr<true, 3, 128, true>();
     if (e != cudaSuccess) return e;
     if (slot >= 0) attr_set[slot] = true;
   }
@@ -1544,7 +1629,8 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
     npoly += f.from_a ? 0u : 1u;
     prm.it[it] = ChainIter{co.a, co.b, co.c, (f.from_a ? kIterFromA : 0u) | (f.fold ? kIterFold : 0u) | (npoly << 8)};
   }
-  // epilogue warps that signal: four; the parameter write that reads W from
+  // epilogue warps that signal: four (three pieces: eight, half the columns
+  // each, for the registers of their sums); the parameter write that reads W from
   // global memory (last APPLY, a not folded) has a launch of its own with eight
   const bool last_fused = c.fuse != nullptr && q1 == 3 * c.steps;
   const bool global_w = last_fused && !(prm.it[c.steps - 1].mode & kIterFold);
@@ -1554,7 +1640,7 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
     return e == cudaSuccess ? launch_ns_chain(c, q1 - 1, q1, st) : e;
   }
   if (last_fused) prm.fuse = *c.fuse;
-  const int base_epi = 4;
+  const int base_epi = c.pieces == 1 ? 4 : kEpiWarps;
   prm.nepi = global_w ? kEpiWarps : base_epi;
   prm.part_sig = 2u * (uint32_t)base_epi;
   prm.sig = c.pieces == 1 ? 2u : prm.part_sig;
@@ -1565,6 +1651,8 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
   const int grid = 2 * c.npairs;
   const bool split = c.ntargets > 0;
   count_launch();
+  if (c.pieces == 3 && c.promote)
+    return split ? launch_chain<true, 3, 128, true>(prm, grid, st) : launch_chain<false, 3, 128, true>(prm, grid, st);
   if (c.pieces == 3)
     return split ? launch_chain<true, 3, 128>(prm, grid, st) : launch_chain<false, 3, 128>(prm, grid, st);
   if (c.bn == 128)

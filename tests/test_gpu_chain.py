@@ -118,3 +118,53 @@ def test_ragged_rows_step(shape, dtype, precision):
     bound = tau * np.linalg.norm(upd) + 2 * ulp * np.linalg.norm(want)
     assert np.linalg.norm(stored_values(p) - want) <= bound
     opt.close()
+
+
+# Full-fp32 mode around the choice of its path (256 rows with the quintic, 320
+# with a table whose |a| reaches 8.5), and on the CUDA cores: one 64-wide tile
+# and just past it, tiles cut along K, 128-wide tiles
+@pytest.mark.parametrize("shape", [(255, 600), (256, 600), (600, 256), (319, 700), (700, 320), (2, 64), (65, 64),
+                                   (64, 5000), (250, 9000), (1000, 1024)])
+def test_full_fp32_msign(shape):
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    from paper_2605_19811_gb300.ns_coeffs import polar_express
+    xh = host_tensor(synth.draw_matrix(shape, seed=shape[0]), "f32")
+    x = stored_values(xh)
+    assert rel_fro(_msign(xh, 0), O.ns_polynomial(x, 5, *QUINTIC, 1e-7)) <= 1e-5
+    if min(shape) >= 255:
+        table = polar_express(5)
+        out = torch.empty(shape, device="cuda")
+        L.msign_ns_coeffs(xh.cuda(), out, table, precision=0)
+        want = O.ns_polynomial_schedule(x, table, 1e-7)
+        # 1e-5 for the quintic, scaled by how much more the table amplifies
+        # fp32 storage on this input (the storage-modelled oracle; about 2)
+        d = rel_fro(O.ns_polynomial_schedule_storage(x, table, 1e-7, "f32"), want)
+        dq = rel_fro(O.ns_polynomial_schedule_storage(x, (QUINTIC,) * 5, 1e-7, "f32"), O.ns_polynomial(x, 5, *QUINTIC, 1e-7))
+        assert rel_fro(stored_values(out), want) <= 1e-5 * max(1.0, d / dq)
+    got = torch.empty(shape, device="cuda")
+    L.msign_ns_noalloc(xh.cuda(), got, precision=0)   # CUDA cores at every size
+    assert rel_fro(stored_values(got), O.ns_polynomial(x, 5, *QUINTIC, 1e-7)) <= 1e-5
+
+
+def test_full_fp32_falls_back_without_the_workspace(monkeypatch):
+    """No room for the three-piece workspace (injected): lm_create takes the
+    CUDA-core path, with a workspace of its own size and the same step."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    shapes = [(320, 512), (512, 320)]
+    g = [host_tensor(x, "f32").cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=0)]
+    out = []
+    for fault in (None, "oom_f32tc"):
+        if fault:
+            monkeypatch.setenv("LM_FAULT", fault)
+        params = [host_tensor(w, "f32").cuda() for w in synth.init_weights(shapes, seed=1)]
+        opt = L.LionMuon(params, period=1, ns_precision=0)
+        opt.step(g, 0)
+        torch.cuda.synchronize()
+        assert opt.status() == 0
+        out.append(([stored_values(p) for p in params], opt.workspace_bytes()))
+        opt.close()
+    assert out[1][1] != out[0][1]
+    for a, b in zip(out[0][0], out[1][0]):
+        assert rel_fro(a, b) <= 1e-6   # the update is 3% of W, both NS within 1e-5
