@@ -269,6 +269,11 @@ int sm_count() {
 // accumulator.  Measured on a 720M-set Muon step: the largest direction error
 // 2.5e-5 at 96 blocks, 1.2e-5 at 48, 8.8e-6 at 32, 8.4e-6 at 24.
 constexpr int kGramCapF32TC = 24;
+// K blocks that cutting a Gram tile has to save in a small batch: writing the
+// parts, waiting for them and summing them takes about 7 us more than writing a
+// whole tile, a K block of a 128-column tile 0.14 us (six piece products: 0.8).
+constexpr int kMaskedGramPart = 200;   // longest Gram part of a large masked batch (K blocks)
+constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
 constexpr uint64_t kRingWaitNs = 2000000000ull;   // the power-iteration ring's waits: 2 s unless set shorter
 
 struct LionTable {
@@ -501,7 +506,7 @@ struct NsLayout {
 // sums).
 static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng, std::vector<NsTile>& t, int tile,
                              int kslice, int workers, std::vector<std::array<int, 6>>& targets, int& nparts_total,
-                             int kcap = 0) {
+                             int kcap, int worth, bool masked) {
   std::vector<int64_t> blocks(ng), len(ng);
   int64_t total = 0, longest = 0;
   for (int g = 0; g < ng; ++g) {
@@ -524,13 +529,24 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
       if (n <= workers) break;
     }
   }
-  const int64_t keep = avg < 32 ? std::max<int64_t>(2 * avg, part) : 2 * avg;   // tiles up to this length stay whole
+  int64_t keep = avg < 32 ? std::max<int64_t>(2 * avg, part) : 2 * avg;   // tiles up to this length stay whole
+  // Under the stable-rank mask a few matrices share the pairs, and in a large
+  // batch a whole embedding tile (786 blocks against a share of 305 on the 355M-
+  // shaped set with a third of the matrices selected) would set the length of
+  // the phase: no part longer than kMaskedGramPart (GRAM 298 -> 150 us per
+  // iteration there).  Without a mask it gains nothing (720M-shaped set: 1%
+  // slower for the summing).
+  if (masked && avg >= 32) {
+    keep = std::min<int64_t>(keep, kMaskedGramPart);
+    part = std::min<int64_t>(part, kMaskedGramPart);
+  }
   if (kcap > 0) part = std::min<int64_t>(part, kcap);
   std::vector<char> whole(ng, 0);
   int64_t planned = 0;   // part numbers are 16 bits (a block may be two tiles wide)
   for (int g = 0; g < ng; ++g) {
     const int64_t n = 2 * blocks[g] * std::min<int64_t>(64, (len[g] + part - 1) / part);
-    whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || planned + n > 65535;
+    whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || planned + n > 65535 ||
+               (kcap <= 0 && avg < 32 && len[g] - part < worth);
     if (!whole[g]) planned += n;
   }
   std::vector<NsTile> out;
@@ -632,7 +648,7 @@ static size_t ns_clear_bytes(int nmat, int ntargets) {
 // two blocks left (bf16 operands).
 static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Arena& ar, Arena& buf, NsLayout& L,
                       std::vector<NsBatch>& batches, int pieces = 1, int tiles_mode = 0, bool masked = false,
-                      bool narrow_ok = true) {
+                      bool narrow_ok = true, bool promote = false) {
   const size_t es = dtype_size(xdt) * (size_t)pieces;
   for (auto& g : groups) {
     const size_t xb = (size_t)g.count * g.s_pad * g.l_pad * es;
@@ -677,7 +693,7 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
     if (xdt == LM_BF16) {
       // three-piece mode: no fp32 accumulation over more than kGramCapF32TC K blocks
       split_gram_tiles(groups, g0, b.ng, lists[NS_GRAM], kTcBM, kTcBK, tc_max_pairs(), targets, nparts,
-                       pieces == 3 ? kGramCapF32TC : 0);
+                       pieces == 3 && !promote ? kGramCapF32TC : 0, pieces == 3 ? kSplitWorthF32 : kSplitWorth, masked);
     } else {
       for (int ph = 0; ph < 3; ++ph) {
         const int parts = split_simt_tiles(groups, g0, ph, b.simt_tile[ph], lists[ph]);
@@ -1332,7 +1348,7 @@ static lm_status create_state(const lm_tensor* params, int n, const lm_config* c
                          s->ns.pieces == 3;
   NsLayout L;
   layout_ns(s->ns.groups, s->ns.xdt, s->nmat, ar, buf, L, s->ns.batches, s->ns.pieces, env_tiles_mode(),
-            cfg->schedule == LM_SCHEDULE_STABLE_RANK, narrow_ok);
+            cfg->schedule == LM_SCHEDULE_STABLE_RANK, narrow_ok, s->ns.promote);
   s->ns.pdl = !env_is("LM_PDL", "0");
   s->ns.wait_ns = env_wait_limit_ns();
   const size_t off_mats = ar.add((size_t)std::max(s->nmat, 1) * sizeof(MatDesc));
@@ -2090,7 +2106,7 @@ static lm_status msign_run(const lm_tensor* in, lm_tensor* out, int steps, const
   plan_groups({{in->rows, in->cols}}, E.xdt, E.groups, members);
   Arena ar, buf;
   NsLayout L;
-  layout_ns(E.groups, E.xdt, 1, ar, buf, L, E.batches, E.pieces, env_tiles_mode());
+  layout_ns(E.groups, E.xdt, 1, ar, buf, L, E.batches, E.pieces, env_tiles_mode(), false, true, E.promote);
   E.pdl = !env_is("LM_PDL", "0");
   E.fold = !env_is("LM_NS_FOLD", "0");
   E.wait_ns = env_wait_limit_ns();
