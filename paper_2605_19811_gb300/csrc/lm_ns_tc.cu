@@ -1079,7 +1079,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       bool ok = true;
       // three pieces: half the tile's columns per warp; the main products of
       // each K block, added in block order
-      float sum[kP == 3 ? 2 : 1][32];
+      float sum[kPromo ? 2 : 1][kPromo ? 32 : 1];
       if constexpr (kPromo) {
         const int nk = phase != NS_GRAM ? g.s_pad / BK : (t.kb1 != 0 ? (int)t.kb1 - (int)t.kb0 : g.l_pad / BK);
         const uint32_t main0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * kBN + half0 * (kBN / 2));
@@ -1147,52 +1147,63 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         const __nv_bfloat16* aux = static_cast<const __nv_bfloat16*>(phase == NS_POLY ? g.A : g.X[cur]);
         __nv_bfloat16* out = static_cast<__nv_bfloat16*>(phase == NS_GRAM ? g.A : (phase == NS_POLY ? g.B : g.X[cur ^ 1]));
         float* out_f32 = (phase == NS_APPLY && p.final_f32 && it == p.steps - 1) ? static_cast<float*>(g.Xf) : nullptr;
+        // one 16-column chunk, columns [c0, c0 + 16) of the tile
+        auto emit = [&](const float (&x)[16], int c0) {
+          const int j = t.tn * kBN + c0;
+          if (!warp_in || j >= jmax) return;   // beyond the padded matrix
+          if (split)
+            split_chunk(x, p.split_ws + (size_t)(t.slot - 1) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN + c0,
+                        nscale, i < nrows, ncols - j);
+          else
+            piece_chunk(x, phase, co, nscale, kacc, aux, out, out_f32, plane,
+                        (size_t)t.mat * msize + (size_t)r0 * ld + j, ld, i < nrows, j, ncols, lane);
+        };
+        // Chunks go through one loop body (unrolled, the copies ran at the pace
+        // of instruction fetch: 7 us per tile).
+        if constexpr (kPromo) {   // half the columns: add the cross products, move the sums down between chunks
+          const int cc = half0 * (kBN / 2);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {   // this warp's 32-column chunks: add the cross products
-          uint32_t rc[32];
-          const uint32_t at = acc0 + (uint32_t)(half0 * (kBN / 2) + c * 32);
-          __syncwarp();   // tcgen05.ld is warp-collective: reconverge first
-          if constexpr (!kPromo) {
-            uint32_t rm[32];
-            tmem_ld32_async(at, rm);
-            tmem_ld32_async(at + (uint32_t)kBN, rc);
-            tmem_ld_wait(rm);
+          for (int c = 0; c < 2; ++c) {
+            uint32_t rc[32];
+            __syncwarp();   // tcgen05.ld is warp-collective: reconverge first
+            tmem_ld32_async(acc0 + (uint32_t)(cc + c * 32), rc);
+            tmem_ld_wait(rc);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) sum[c][e] = __uint_as_float(rm[e]);
-          } else {
-            tmem_ld32_async(at, rc);
+            for (int e = 0; e < 32; ++e) sum[c][e] += __uint_as_float(rc[e]);
           }
-          tmem_ld_wait(rc);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) sum[c][e] += __uint_as_float(rc[e]);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
-        // one loop body for the warp's four 16-column chunks, the sums moved down
-        // between them (unrolled, the four copies ran at the pace of instruction
-        // fetch: 7 us per tile)
-        const int cc = half0 * (kBN / 2), j0 = t.tn * kBN + cc;
-        float* wrow = split ? p.split_ws + (size_t)(t.slot - 1) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN + cc
-                            : nullptr;
-        const size_t base = (size_t)t.mat * msize + (size_t)r0 * ld + j0;   // row r0 = this warp's first
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
 #pragma unroll 1
-        for (int h = 0; h < 4; ++h) {
-          float x[16];
+          for (int h = 0; h < 4; ++h) {
+            float x[16];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) x[e] = sum[0][e];
-          const int j = j0 + 16 * h;
-          if (warp_in && j < jmax) {   // inside the padded matrix
-            if (split) split_chunk(x, wrow + 16 * h, nscale, i < nrows, ncols - j);
-            else piece_chunk(x, phase, co, nscale, kacc, aux, out, out_f32, plane, base + 16 * h, ld, i < nrows, j,
-                             ncols, lane);
-          }
+            for (int e = 0; e < 16; ++e) x[e] = sum[0][e];
+            emit(x, cc + 16 * h);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            sum[0][e] = sum[0][16 + e];
-            sum[0][16 + e] = sum[1][e];
-            sum[1][e] = sum[1][16 + e];
+            for (int e = 0; e < 16; ++e) {
+              sum[0][e] = sum[0][16 + e];
+              sum[0][16 + e] = sum[1][e];
+              sum[1][e] = sum[1][16 + e];
+            }
           }
+        } else {   // all columns (four epilogue warps): main + cross accumulators
+#pragma unroll 1
+          for (int ch = 0; ch < kBN / 16; ++ch) {
+            uint32_t rm[16], rc[16];
+            __syncwarp();
+            tmem_ld16_async(acc0 + (uint32_t)(ch * 16), rm);
+            tmem_ld16_async(acc0 + (uint32_t)(kBN + ch * 16), rc);
+            tmem_ld_wait(rm);
+            tmem_ld_wait(rc);
+            float x[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(rm[e]) + __uint_as_float(rc[e]);
+            emit(x, ch * 16);
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(ab == 0 ? acc_empty0 : acc_empty1);
         }
       } else if (split) {
         // partial Gram product of a split tile: its own fp32 workspace tile
@@ -1635,8 +1646,8 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
     npoly += f.from_a ? 0u : 1u;
     prm.it[it] = ChainIter{co.a, co.b, co.c, (f.from_a ? kIterFromA : 0u) | (f.fold ? kIterFold : 0u) | (npoly << 8)};
   }
-  // epilogue warps that signal: four (three pieces: eight, half the columns
-  // each, for the registers of their sums); the parameter write that reads W from
+  // epilogue warps that signal: four (with register sums eight, half the columns
+  // each); the parameter write that reads W from
   // global memory (last APPLY, a not folded) has a launch of its own with eight
   const bool last_fused = c.fuse != nullptr && q1 == 3 * c.steps;
   const bool global_w = last_fused && !(prm.it[c.steps - 1].mode & kIterFold);
@@ -1646,7 +1657,7 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
     return e == cudaSuccess ? launch_ns_chain(c, q1 - 1, q1, st) : e;
   }
   if (last_fused) prm.fuse = *c.fuse;
-  const int base_epi = c.pieces == 1 ? 4 : kEpiWarps;
+  const int base_epi = c.pieces == 3 && c.promote ? kEpiWarps : 4;
   prm.nepi = global_w ? kEpiWarps : base_epi;
   prm.part_sig = 2u * (uint32_t)base_epi;
   prm.sig = c.pieces == 1 ? 2u : prm.part_sig;
