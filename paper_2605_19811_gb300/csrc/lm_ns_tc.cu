@@ -303,6 +303,14 @@ __device__ __forceinline__ void split3(float v, float& h, float& m, float& l) {
   m = __bfloat162float(__float2bfloat16_rn(r1));
   l = r1 - m;
 }
+// The same for a pair of values, packed: the conversion to bf16 packs, and the
+// halves are what is subtracted.
+__device__ __forceinline__ void split3_pair(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+  h = pack_bf2(a, b);
+  const float ra = a - bf_lo(h), rb = b - bf_hi(h);
+  m = pack_bf2(ra, rb);
+  l = pack_bf2(ra - bf_lo(m), rb - bf_hi(m));
+}
 // Epilogue of one 32 x 16 chunk (rows r0 .. r0 + 31, one per lane; columns
 // j0 ..) with three-piece operands; aux values and results go through global
 // memory in whole 32-byte sectors: lanes 2m and 2m + 1 access the two halves of
@@ -312,33 +320,47 @@ __device__ __forceinline__ void split3(float v, float& h, float& m, float& l) {
 //   aux: the A (POLY) or X (APPLY) element, hi + mid + lo; out: the result's
 //   pieces, or fp32 in out_f32 (last APPLY).  base: element (r0, j0) of the
 //   matrix in plane 0; ld: row length; plane: elements per piece.
-template <typename Co>
+struct AuxPieces {
+  uint4 v[2][3];   // this lane's halves of rows 2m and 2m + 1, per plane
+};
+__device__ __forceinline__ void aux_load(AuxPieces& a, const __nv_bfloat16* aux, size_t plane, size_t base, size_t ld,
+                                         int lane) {
+  const size_t off0 = base + (size_t)(lane & ~1) * ld + ((lane & 1) ? 8 : 0);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int q = 0; q < 3; ++q)   // through L2: another SM may have written the tile in this launch
+      a.v[k][q] = __ldcg(reinterpret_cast<const uint4*>(aux + q * plane + off0 + (size_t)k * ld));
+}
+// kAhead: a holds the chunk's aux values (not GRAM) and next, if next_ok, is the
+// base of the chunk after it, whose aux values are loaded into a while this one
+// is combined; without (register sums: no registers to spare) they are loaded
+// here.
+template <bool kAhead, typename Co>
 __device__ __forceinline__ void piece_chunk(const float (&acc)[16], int phase, const Co& co, float nscale,
-                                            float kacc,
+                                            float kacc, AuxPieces& a,
                                             const __nv_bfloat16* aux, __nv_bfloat16* out, float* out_f32,
                                             size_t plane, size_t base, size_t ld, bool row_ok, int j0, int ncols,
-                                            int lane) {
+                                            bool next_ok, size_t next, int lane) {
   const bool odd = lane & 1;
   const size_t off0 = base + (size_t)(lane & ~1) * ld + (odd ? 8 : 0);   // this lane's half of row 2m
   float v[16];
   if (phase != NS_GRAM) {
     float h[2][8];   // this lane's halves of rows 2m and 2m + 1
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-#pragma unroll
-      for (int t = 0; t < 8; ++t) h[k][t] = 0.f;
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        // through L2: another SM may have written the tile in this launch
-        const uint4 a4 = __ldcg(reinterpret_cast<const uint4*>(aux + q * plane + off0 + (size_t)k * ld));
+        const uint4 a4 = kAhead ? a.v[k][q]
+                                : __ldcg(reinterpret_cast<const uint4*>(aux + q * plane + off0 + (size_t)k * ld));
         const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          h[k][2 * e] += bf_lo(aw[e]);
-          h[k][2 * e + 1] += bf_hi(aw[e]);
+          h[k][2 * e] = q == 0 ? bf_lo(aw[e]) : h[k][2 * e] + bf_lo(aw[e]);
+          h[k][2 * e + 1] = q == 0 ? bf_hi(aw[e]) : h[k][2 * e + 1] + bf_hi(aw[e]);
         }
       }
-    }
+    if (kAhead && next_ok) aux_load(a, aux, plane, next, ld, lane);
 #pragma unroll
     for (int t = 0; t < 8; ++t) {   // an even lane owns row 2m, an odd one row 2m + 1
       const float got = __shfl_xor_sync(0xffffffffu, odd ? h[0][t] : h[1][t], 1);
@@ -372,14 +394,7 @@ __device__ __forceinline__ void piece_chunk(const float (&acc)[16], int phase, c
     }
     uint32_t w[3][4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float h0, m0, l0, h1, m1, l1;
-      split3(h[k][2 * e], h0, m0, l0);
-      split3(h[k][2 * e + 1], h1, m1, l1);
-      w[0][e] = pack_bf2(h0, h1);
-      w[1][e] = pack_bf2(m0, m1);
-      w[2][e] = pack_bf2(l0, l1);
-    }
+    for (int e = 0; e < 4; ++e) split3_pair(h[k][2 * e], h[k][2 * e + 1], w[0][e], w[1][e], w[2][e]);
 #pragma unroll
     for (int q = 0; q < 3; ++q)
       *reinterpret_cast<uint4*>(out + q * plane + off) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
@@ -1147,16 +1162,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         const __nv_bfloat16* aux = static_cast<const __nv_bfloat16*>(phase == NS_POLY ? g.A : g.X[cur]);
         __nv_bfloat16* out = static_cast<__nv_bfloat16*>(phase == NS_GRAM ? g.A : (phase == NS_POLY ? g.B : g.X[cur ^ 1]));
         float* out_f32 = (phase == NS_APPLY && p.final_f32 && it == p.steps - 1) ? static_cast<float*>(g.Xf) : nullptr;
-        // one 16-column chunk, columns [c0, c0 + 16) of the tile
+        // One 16-column chunk, columns [c0, c0 + 16) of the tile, next c0 + 16
+        // of this warp's columns up to c1.  A chunk's aux values are loaded one
+        // chunk ahead, the first before the accumulators are read.
+        const size_t tile0 = (size_t)t.mat * msize + (size_t)r0 * ld + (size_t)t.tn * kBN;
+        const int first = kPromo ? half0 * (kBN / 2) : 0, c1 = kPromo ? first + kBN / 2 : kBN;
+        auto inside = [&](int c0) { return warp_in && c0 < c1 && t.tn * kBN + c0 < jmax; };   // the padded matrix
+        AuxPieces ap;
+        if (!kPromo && phase != NS_GRAM && inside(first)) aux_load(ap, aux, plane, tile0 + first, ld, lane);
         auto emit = [&](const float (&x)[16], int c0) {
           const int j = t.tn * kBN + c0;
-          if (!warp_in || j >= jmax) return;   // beyond the padded matrix
+          if (!inside(c0)) return;
           if (split)
             split_chunk(x, p.split_ws + (size_t)(t.slot - 1) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN + c0,
                         nscale, i < nrows, ncols - j);
           else
-            piece_chunk(x, phase, co, nscale, kacc, aux, out, out_f32, plane,
-                        (size_t)t.mat * msize + (size_t)r0 * ld + j, ld, i < nrows, j, ncols, lane);
+            piece_chunk<!kPromo>(x, phase, co, nscale, kacc, ap, aux, out, out_f32, plane, tile0 + c0, ld, i < nrows, j, ncols,
+                        !kPromo && inside(c0 + 16), tile0 + c0 + 16, lane);
         };
         // Chunks go through one loop body (unrolled, the copies ran at the pace
         // of instruction fetch: 7 us per tile).
