@@ -239,7 +239,8 @@ struct Arena {
 //                      they fit, run by the wide-tile kernel; the default
 //                      (or LM_NS_TILES=narrow) is one-block tiles.  The
 //                      results are the same bit for bit
-//   LM_PDL=0           no programmatic dependent launch between NS launches
+//   LM_PDL=0           no programmatic dependent launch between the
+//                      wide-tile kernel's launches
 //   LM_NS_FOLD=0       keep a X as a separate term of APPLY instead of folding
 //                      a into B's diagonal
 //   LM_WAIT_LIMIT_NS=n limit of every bounded device wait (default 5 s; a
@@ -269,10 +270,12 @@ int sm_count() {
 // accumulator.  Measured on a 720M-set Muon step: the largest direction error
 // 2.5e-5 at 96 blocks, 1.2e-5 at 48, 8.8e-6 at 32, 8.4e-6 at 24.
 constexpr int kGramCapF32TC = 24;
+constexpr int kMaskedGramPart = 200;   // longest Gram part of a large masked batch (K blocks)
 // K blocks that cutting a Gram tile has to save in a small batch: writing the
 // parts, waiting for them and summing them takes about 7 us more than writing a
 // whole tile, a K block of a 128-column tile 0.14 us (six piece products: 0.8).
-constexpr int kMaskedGramPart = 200;   // longest Gram part of a large masked batch (K blocks)
+// 2-layer d = 128 Muon step 126 -> 109 us (no cuts now); 24 instead of 48: one
+// d = 768 layer 239 us against 230.
 constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
 constexpr uint64_t kRingWaitNs = 2000000000ull;   // the power-iteration ring's waits: 2 s unless set shorter
 
@@ -534,8 +537,8 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
   // batch a whole embedding tile (786 blocks against a share of 305 on the 355M-
   // shaped set with a third of the matrices selected) would set the length of
   // the phase: no part longer than kMaskedGramPart (GRAM 298 -> 150 us per
-  // iteration there).  Without a mask it gains nothing (720M-shaped set: 1%
-  // slower for the summing).
+  // iteration there, the step 4658 -> 3957 us).  Without a mask it gains
+  // nothing (720M-shaped set: 1% slower for the summing).
   if (masked && avg >= 32) {
     keep = std::min<int64_t>(keep, kMaskedGramPart);
     part = std::min<int64_t>(part, kMaskedGramPart);
@@ -901,7 +904,8 @@ static cudaError_t timed(Profiler* P, int fam, cudaStream_t st, F&& f) {
 // far with the quintic and the degree-5 minimax table, at 256 0.26 to 0.63
 // with the quintic but up to 1.2 with the table (whose first |a| is 8.5);
 // narrower matrices go either way (130 x 200: 0.37 to 6).  An msign of 1024 x
-// 1024 takes 516 us there against 1026 us.
+// 1024 takes 465 us there against 1026 us, a step of the 124M-shaped set (P = 2)
+// 6.0 ms against 17.4.
 static bool f32_on_tensor_cores(const std::vector<std::pair<int64_t, int64_t>>& shapes, const std::vector<NsCoeffs>& co) {
   int64_t least = 320;
   bool small_a = true;

@@ -21,8 +21,9 @@
 // block that finishes last adds the parts in order and writes the result, so
 // the sum does not depend on timing and nothing waits.
 // Same box, against 128-wide tiles only and a summing launch after each split
-// Gram: tiny fp32 set (256 x 256 to 256 x 1024) 541 -> 314 us per Muon step,
-// msign of 1024 x 1024 1497 -> 1026 us.
+// Gram: tiny fp32 set (256 x 256 to 256 x 1024, which now runs on the tensor
+// cores) 541 -> 314 us per Muon step, msign of 1024 x 1024 1497 -> 1026 us,
+// lm_msign_ns_noalloc of 1024 x 1024 1795 -> 917 us.
 #include "lm_internal.h"
 
 namespace lm {

@@ -28,10 +28,10 @@
 // for the counter, 3.3 us of MMAs (K = 768, half of that on 128 columns), 1.3 us
 // for the epilogue, 1.5 us until the stores are complete and counted.
 // Measured on one box against one launch per phase with the epilogue warps
-// storing and waiting: 124M-shaped Muon step 1731 -> 1531 us, small sets
-// (2 layers, d = 128) 195 -> 129 us, one d = 768 layer from a graph 335 -> 236
-// us, 720M-shaped set the same within 1 % (power-capped), three-piece 4-layer
-// set 8041 -> 7626 us.
+// storing and waiting: 124M-shaped Muon step 1720 -> 1518 us, small sets
+// (2 layers, d = 128) 193 -> 109 us, one d = 768 layer from a graph 338 -> 231
+// us, 720M-shaped set the same within 1% (power-capped), three-piece 4-layer
+// d = 1280 set 8030 -> 7440 us.
 //
 // CTA roles (384 threads, one CTA per SM; 12 warps, three per sub-partition):
 //   warp 0    TMA producer (one lane), smem ring (TcLayout); both CTAs' copies
@@ -40,9 +40,11 @@
 //   warps 2-9 epilogue: tcgen05.ld from TMEM, fused polynomial combination,
 //             results written into shared memory (over the aux tile).  Warps
 //             2-5 (one per TMEM lane quadrant and SM sub-partition) cover the
-//             whole tile; warps 6-9 work only in a launch whose parameter
-//             write reads W from global memory (latency-bound), and all eight
-//             sum the split-K parts.  Eight epilogue warps elsewhere measured
+//             whole tile; warps 6-9 work only where the main products are
+//             summed in registers (kPromo, half the columns each) and in a
+//             launch whose parameter write reads W from global memory
+//             (latency-bound), and all eight sum the split-K parts.  Eight
+//             epilogue warps elsewhere measured
 //             1 to 4% slower per Muon step on the d = 768 and 1280 sets: two of
 //             them share each sub-partition's issue slots with the producer or
 //             the MMA issuer.
@@ -232,7 +234,7 @@ __device__ __forceinline__ bool produce_range(ProducerRing<TcLayout<kP, kBN>::kS
 // 1.4e-6 against 1.6e-6 to 3.3e-6; dropping no product at all, eight of them,
 // changes nothing).  Its cost: the warps that hold the sums cannot go on adding
 // while they write a tile out, so the MMAs of the next tile wait (4-layer d =
-// 1280 set: 10.7 ms per Muon step against 7.6 without).
+// 1280 set: 10.7 ms per Muon step against 7.4-7.6 without).
 // Main products: per K block n, accumulator n & 1; mfull: the block's four MMAs
 // are done (both CTAs), mempty: every epilogue warp has read it.
 struct MainRing {
