@@ -277,6 +277,16 @@ constexpr int kMaskedGramPart = 200;   // longest Gram part of a large masked ba
 // 2-layer d = 128 Muon step 126 -> 109 us (no cuts now); 24 instead of 48: one
 // d = 768 layer 239 us against 230.
 constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
+// K blocks per CTA pair and iteration from which a batch runs one launch per
+// phase instead of one for the whole chain.  Such a batch works under the power
+// cap, where the chain's polls and its gapless run cost clocks as well as they
+// save gaps (2% of 2.1 ms an iteration): 720M-shaped set (6800 blocks), a Muon
+// and a Lion step sustained on three GPUs against the launches of the kernel
+// without the chain: one launch +1.1, -0.6 and -2%, a launch per phase +0.3 and
+// +0.4% (two of them); three-piece 4-layer d = 1280 set (4200) 7460 us in one
+// launch, 7370 per phase.  Below, one launch wins: 355M-shaped set (2600) 4.83 ms
+// per Muon step against 5.00, 124M-shaped 1515 us against 1672.
+constexpr int kPhaseLaunchBlocks = 4096;
 constexpr uint64_t kRingWaitNs = 2000000000ull;   // the power-iteration ring's waits: 2 s unless set shorter
 
 struct LionTable {
@@ -294,6 +304,7 @@ struct NsBatch {
   bool wide = false;                               // tiles of two 256-column blocks: the wide-tile kernel
   int* offsets[3] = {nullptr, nullptr, nullptr};   // per-pair tile ranges (tensor-core path), NULL: snake order
   int npairs = 0;                                  // CTA pairs (tensor-core path)
+  bool per_phase = false;                          // a launch per phase of the chain (kPhaseLaunchBlocks)
   int bn = kTcBN;                                  // columns of a tile (tensor-core path)
   int simt_tile[3] = {kSimtBM, kSimtBM, kSimtBM};  // tile of each phase (fp32 path)
   NsTile* compact[3] = {nullptr, nullptr, nullptr};   // masked steps: the selected matrices' tiles and their counts
@@ -729,6 +740,7 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
     if (xdt == LM_BF16)
       b.npairs = (int)std::min<size_t>((size_t)tc_max_pairs(),
                                        std::max(lists[0].size(), std::max(lists[1].size(), lists[2].size())));
+    int64_t work = 0;   // of an iteration, in K blocks
     for (int ph = 0; ph < 3; ++ph) {
       std::vector<NsTile>& t = lists[ph];
       std::vector<int> offs;
@@ -739,6 +751,7 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
           const NsGroup& g = groups[g0 + x.group];
           const int nk = (ph == NS_GRAM) ? (x.kb1 != 0 ? x.kb1 - x.kb0 : g.l_pad / kTcBK) : g.s_pad / kTcBK;
           sorted.push_back({(nk + 6) * (x.nh == 2 ? 2 : 1), x});
+          work += sorted.back().first;
         }
         std::stable_sort(sorted.begin(), sorted.end(),
                          [](const std::pair<int, NsTile>& a, const std::pair<int, NsTile>& c) {
@@ -761,6 +774,8 @@ static void layout_ns(std::vector<NsGroup>& groups, lm_dtype xdt, int nmat, Aren
       L.off_offsets.push_back(ar.add(offs.size() * sizeof(int)));
       L.offsets.push_back(std::move(offs));
     }
+    // (six products of half the columns: three times a 256-column block)
+    b.per_phase = !promote && !masked && work * (pieces == 3 ? 3 : 1) >= (int64_t)kPhaseLaunchBlocks * b.npairs;
     L.off_counts.push_back(masked ? ar.add(3 * sizeof(int)) : 0);
     batches.push_back(b);
   }
@@ -978,9 +993,9 @@ static lm_status run_ns(const NsEngine& E, int steps, const NsCoeffs* coeffs, un
       c.active = active;
       c.flags = flags;
       c.wait_ns = E.wait_ns;
-      // one launch for the whole chain; with profiling on, one per phase, so
-      // that every phase has a time of its own
-      if (!profiling(P, st)) {
+      // one launch for the whole chain, or one per phase: for large batches, and
+      // with profiling on, so that every phase has a time of its own
+      if (!profiling(P, st) && !b.per_phase) {
         cudaError_t e = launch_ns_chain(c, 0, 3 * steps, st);
         if (e != cudaSuccess) return cuda_fail(e, "Newton-Schulz launch");
         continue;
