@@ -50,8 +50,9 @@ def parse_args():
     ap.add_argument("--set", default="gpt_720m")
     ap.add_argument("--period", type=int, default=2)
     ap.add_argument("--precision", choices=["bf16", "f32", "f32tc"], default="bf16",
-                    help="NS precision: bf16 tensor cores, fp32 CUDA cores, or fp32 values as three "
-                         "bf16 pieces on the tensor cores")
+                    help="NS precision: bf16 tensor cores; full fp32 (tensor cores with fp32 register "
+                         "sums for wide sets, else CUDA cores); or fp32 values as three bf16 pieces on the "
+                         "tensor cores")
     ap.add_argument("--schedule", choices=["period", "srank"], default="period",
                     help="period: Algorithm 1's fixed P; srank: Appendix G's stable-rank selection")
     ap.add_argument("--srank-alpha", type=float, default=0.01)
@@ -616,6 +617,10 @@ def run_ours(args):
     pk_bf16 = pk_sust if long_region else pk_burst
     bf16_kind = (f"bf16 {'sustained' if long_region else 'burst'} ({ms_total / 1e3:.2f} s timed region), "
                  f"{peak_src}")
+    # fp32 modes on the tensor cores: LM_NS_F32_TC, and LM_F32 where every matrix
+    # is wide enough (256 where all |a| < 4, 320 otherwise)
+    least = 256 if table is None or all(abs(row[0]) < 4 for row in table) else 320
+    pieces = args.precision == "f32tc" or (args.precision == "f32" and min(min(m) for m in ns_mats) >= least)
     roof = None
     if ns_ms > 0 and n_muon > 0:
         achieved = fl / (ns_ms / 1e3) / 1e12
@@ -624,7 +629,7 @@ def run_ours(args):
         if args.precision == "bf16":
             pk = pk_bf16
             bound, kernel, peak_kind = "tensor", "ns_tc_kernel", bf16_kind
-        elif args.precision == "f32tc":
+        elif pieces:
             # six bf16 piece products per fp32 product, on the bf16 tensor pipe
             achieved *= 6
             fl *= 6
@@ -646,7 +651,7 @@ def run_ours(args):
         ph_fl = {"ns_gram": sum(min(a, b) ** 2 * max(a, b) for a, b in ns_mats),
                  "ns_poly": sum(min(a, b) ** 3 for a, b in ns_mats),
                  "ns_apply": sum(2.0 * min(a, b) ** 2 * max(a, b) for a, b in ns_mats)}
-        mult = 6 if args.precision == "f32tc" else 1
+        mult = 6 if pieces else 1
         phases = {}
         for k, f1 in ph_fl.items():
             ms_k, n_k = prof[k]

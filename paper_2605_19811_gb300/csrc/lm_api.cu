@@ -920,7 +920,7 @@ static cudaError_t timed(Profiler* P, int fam, cudaStream_t st, F&& f) {
 // with the quintic but up to 1.2 with the table (whose first |a| is 8.5);
 // narrower matrices go either way (130 x 200: 0.37 to 6).  An msign of 1024 x
 // 1024 takes 465 us there against 1026 us, a step of the 124M-shaped set (P = 2)
-// 6.0 ms against 17.4.
+// 5.1 ms against 17.4.
 static bool f32_on_tensor_cores(const std::vector<std::pair<int64_t, int64_t>>& shapes, const std::vector<NsCoeffs>& co) {
   int64_t least = 320;
   bool small_a = true;

@@ -1,7 +1,8 @@
 // Tensor-core Newton-Schulz chain for sm_103a: tcgen05.mma (bf16 operands,
 // fp32 accumulators in TMEM) on CTA pairs (cta_group::2, one 256-row tile of
 // 256 or 128 columns per pair), operands staged by TMA into 128-byte-swizzled
-// shared memory; one persistent launch runs all phases of all iterations.
+// shared memory; one persistent launch runs all phases of all iterations (large
+// batches: one phase, lm_api.cu says why).
 //
 // Per NS iteration (Section 2, odd-polynomial Newton-Schulz), with the
 // normalisation X / (||G_hat||_F + eps) folded into iteration 0.  A wide
@@ -30,8 +31,9 @@
 // Measured on one box against one launch per phase with the epilogue warps
 // storing and waiting: 124M-shaped Muon step 1720 -> 1518 us, small sets
 // (2 layers, d = 128) 193 -> 109 us, one d = 768 layer from a graph 338 -> 231
-// us, 720M-shaped set the same within 1% (power-capped), three-piece 4-layer
-// d = 1280 set 8030 -> 7440 us.
+// us, three-piece 4-layer d = 1280 set 8030 -> 7460 us; in a launch per phase
+// that set 7380 us, the 720M-shaped set (power-capped) 14.27 -> 14.21 ms for a
+// Muon and a Lion step.
 //
 // CTA roles (384 threads, one CTA per SM; 12 warps, three per sub-partition):
 //   warp 0    TMA producer (one lane), smem ring (TcLayout); both CTAs' copies
