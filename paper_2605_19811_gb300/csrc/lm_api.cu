@@ -1838,6 +1838,9 @@ lm_status lm_step(lm_state* s, const lm_tensor* grads, int n, int64_t t, void* c
   MuonConsts mk = muon_consts(c);
   mk.flags = s->d_flags;
   if (mixed) mk.active = s->d_active;
+  // the vectors' Lion step goes with the momentum launch of their dtype (a launch
+  // of its own with profiling on, so that each family has its time)
+  bool ridden[2] = {false, false};
   if (s->nmat > 0) {
     e = timed(P, LM_KERNEL_OTHER, stream, [&]() {
       return cudaMemsetAsync(s->ns.d_norm2, 0, s->ns.clear_bytes, stream);
@@ -1845,9 +1848,14 @@ lm_status lm_step(lm_state* s, const lm_tensor* grads, int n, int64_t t, void* c
     if (e != cudaSuccess) return cuda_fail(e, "norm reset");
     for (int dt = 0; dt < 2; ++dt) {
       if (s->n_echunks[dt] == 0) continue;
+      LionRide ride;
+      if (!s->adamw && !mixed && s->lion_vec[dt].nchunks > 0 && !profiling(P, stream)) {
+        ride = LionRide{s->lion_vec[dt].tensors, s->lion_vec[dt].chunks, s->lion_vec[dt].nchunks, lk};
+        ridden[dt] = true;
+      }
       e = timed(P, LM_KERNEL_MOMENTUM_NORM, stream, [&]() {
         return launch_momentum_norm(s->ns.pieces == 3 ? LM_F32 : s->ns.xdt, (lm_dtype)dt, s->d_mats,
-                                    s->d_echunks[dt], s->n_echunks[dt], s->d_grads, mk, 0, stream);
+                                    s->d_echunks[dt], s->n_echunks[dt], s->d_grads, mk, 0, stream, ride);
       });
       if (e != cudaSuccess) return cuda_fail(e, "momentum/norm kernel launch");
     }
@@ -1866,7 +1874,7 @@ lm_status lm_step(lm_state* s, const lm_tensor* grads, int n, int64_t t, void* c
     if ((st = run_adamw(s, t, stream)) != LM_OK) return st;
   }
   for (int d = 0; d < 2 && !s->adamw && !mixed; ++d) {
-    if (s->lion_vec[d].nchunks == 0) continue;
+    if (s->lion_vec[d].nchunks == 0 || ridden[d]) continue;
     e = timed(P, LM_KERNEL_LION, stream, [&]() {
       return launch_lion((lm_dtype)d, s->lion_vec[d].tensors, s->lion_vec[d].chunks,
                          s->lion_vec[d].nchunks, s->d_grads, lk, s->lion_grid[d], stream);

@@ -168,3 +168,29 @@ def test_full_fp32_falls_back_without_the_workspace(monkeypatch):
     assert out[1][1] != out[0][1]
     for a, b in zip(out[0][0], out[1][0]):
         assert rel_fro(a, b) <= 1e-6   # the update is 3% of W, both NS within 1e-5
+
+
+# 1-D parameters beside a bf16 matrix: of its dtype they take their Lion step in
+# the momentum launch, of the other in a launch of their own; lengths around a
+# vector of 8 and a chunk of 2048 elements, and many chunks
+@pytest.mark.parametrize("n", [1, 7, 8, 2047, 2048, 2049, 70003])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_vectors_in_the_momentum_launch(n, dtype):
+    """Bit-identical to the Lion kernel (with profiling on the vectors always
+    have its launch)."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    shapes, dtypes = [(96, 200), (1, n), (1, 5)], ["bf16", dtype, "bf16"]
+    got = []
+    for profile in (False, True):
+        params = [host_tensor(w, d).cuda() for w, d in zip(synth.init_weights(shapes, seed=3), dtypes)]
+        opt = L.LionMuon(params, period=1, eta_lion=1e-3, weight_decay=0.1)
+        opt.profile(profile)
+        for t in range(3):
+            gs = synth.draw_grads(shapes, "student_t", seed=4, step=t)
+            opt.step([host_tensor(x, d).cuda() for x, d in zip(gs, dtypes)], t)
+        torch.cuda.synchronize()
+        assert opt.status() == 0
+        got.append([bits(p) for p in params] + [bits(opt.momentum(i)) for i in range(3)])
+    for x, y in zip(*got):
+        np.testing.assert_array_equal(x, y)
