@@ -282,8 +282,8 @@ constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
 // cap, where the chain's polls and its gapless run cost clocks as well as they
 // save gaps (2% of 2.1 ms an iteration): 720M-shaped set (6800 blocks), a Muon
 // and a Lion step sustained on three GPUs against the launches of the kernel
-// without the chain: one launch +1.1, -0.6 and -2%, a launch per phase +0.3 and
-// +0.4% (two of them); three-piece 4-layer d = 1280 set (4200) 7460 us in one
+// without the chain: one launch +1.1, -0.6 and -2%, a launch per phase 0 to
+// +0.5% (four GPUs); three-piece 4-layer d = 1280 set (4200) 7460 us in one
 // launch, 7370 per phase.  Below, one launch wins: 355M-shaped set (2600) 4.83 ms
 // per Muon step against 5.00, 124M-shaped 1515 us against 1672.
 constexpr int kPhaseLaunchBlocks = 4096;

@@ -32,8 +32,8 @@
 // storing and waiting: 124M-shaped Muon step 1720 -> 1518 us, small sets
 // (2 layers, d = 128) 193 -> 109 us, one d = 768 layer from a graph 338 -> 231
 // us, three-piece 4-layer d = 1280 set 8030 -> 7460 us; in a launch per phase
-// that set 7380 us, the 720M-shaped set (power-capped) 14.27 -> 14.21 ms for a
-// Muon and a Lion step.
+// that set 7300-7380 us, the 720M-shaped set (power-capped) 14.2-14.3 ms for a
+// Muon and a Lion step both ways.
 //
 // CTA roles (384 threads, one CTA per SM; 12 warps, three per sub-partition):
 //   warp 0    TMA producer (one lane), smem ring (TcLayout); both CTAs' copies
