@@ -1093,8 +1093,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       const MatDesc* fd = fused ? &p.fuse.mats[g.first_mat + t.mat] : nullptr;
       const bool global_w = kP == 1 && fused && !fold;
       // a tile whose epilogue starts after a give-up was recorded leaves W alone
+      // (another matrix's non-finite norm, in the same word, does not stop it)
       const unsigned flags_now = global_w && lane == 0 ? *reinterpret_cast<volatile unsigned*>(p.flags) : 0u;
-      const bool write_w = global_w && __shfl_sync(0xffffffffu, flags_now, 0) == 0u;
+      const bool write_w = global_w && (__shfl_sync(0xffffffffu, flags_now, 0) & LM_FLAG_TIMEOUT) == 0u;
       bool ok = true;
       // three pieces: half the tile's columns per warp; the main products of
       // each K block, added in block order

@@ -409,8 +409,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const bool fused = phase == NS_APPLY && p.fuse.mats != nullptr;
       const MatDesc* fd = fused ? &p.fuse.mats[g.first_mat + t.mat] : nullptr;
       // a tile whose epilogue starts after a give-up was recorded leaves W alone
+      // (another matrix's non-finite norm, in the same word, does not stop it)
       const unsigned flags_now = fused && lane == 0 ? *reinterpret_cast<volatile unsigned*>(p.flags) : 0u;
-      const bool write_w = fused && __shfl_sync(0xffffffffu, flags_now, 0) == 0u;
+      const bool write_w = fused && (__shfl_sync(0xffffffffu, flags_now, 0) & LM_FLAG_TIMEOUT) == 0u;
       float nscale = 1.f;
       if (p.iter == 0) {
         const float n = (float)sqrt(p.norm2[g.first_mat + t.mat]) + p.co.eps;

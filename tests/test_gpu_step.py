@@ -370,3 +370,36 @@ def test_coefficient_table_rejected_when_not_finite():
     with pytest.raises(L.LionMuonError) as e:
         L.LionMuon(p, ns_coeffs=[(1.0, 0.0, 0.0), (float("inf"), 0.0, 0.0)])
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("env,cfg", [
+    ({}, {}),                                                     # the write on the W tile (a folded)
+    ({"LM_NS_FOLD": "0"}, {}),                                    # the write through global memory
+    ({}, dict(ns_coeffs=((3.4445, -4.775, 2.0315), (1.5, -0.5, 0.0)))),   # the same, last iteration a cubic
+    ({"LM_NS_TILES": "wide"}, {}),                                # the two-block tile kernel
+    ({}, dict(ns_precision=2))])                                  # finalize_kernel
+def test_nonfinite_matrix_leaves_the_others_alone(env, cfg, monkeypatch):
+    """An Inf in one matrix's gradient raises LM_FLAG_NONFINITE and spoils that
+    matrix only: the others are updated, in that step and in those after it
+    (the flag is still set), exactly as without the Inf."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    shapes = [(256, 512), (768, 768), (512, 256), (768, 768)]
+    bad, runs = 1, []
+    for inf in (False, True):
+        params = [host_tensor(w, "bf16").cuda() for w in synth.init_weights(shapes, seed=1)]
+        opt = L.LionMuon(params, period=1, **cfg)
+        for t in range(3):
+            g = [host_tensor(x, "bf16").cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=t)]
+            if inf and t == 0:
+                g[bad][5, 7] = float("inf")
+            opt.step(g, t)
+        torch.cuda.synchronize()
+        flags = opt.status()
+        assert not flags & L.LM_FLAG_TIMEOUT and bool(flags & L.LM_FLAG_NONFINITE) == inf
+        runs.append([bits(x) for i in range(len(shapes)) if i != bad for x in (params[i], opt.momentum(i))])
+        opt.close()
+    for a, b in zip(*runs):
+        np.testing.assert_array_equal(a, b)
