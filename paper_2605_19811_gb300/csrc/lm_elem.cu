@@ -301,7 +301,9 @@ constexpr int kFinVec = 2, kFinCtas = 3;
 // vectors with the rounding error of every addition carried along (Knuth's
 // two-sum), so the norm does not depend on how elements fall into chunks (ranks
 // of a sharded set chunk differently) and costs no fp64 arithmetic per vector
-// (this GPU's fp64 rate is a small fraction of its fp32 rate).
+// (this GPU's fp64 rate is a small fraction of its fp32 rate).  Once s is
+// infinite (squares beyond fp32) the error terms are Inf - Inf, and the total
+// is s alone.
 struct SquareSum {
   float s = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float a) {
@@ -310,6 +312,7 @@ struct SquareSum {
     lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b)));
     s = t;
   }
+  __device__ __forceinline__ double total() const { return isfinite(s) ? (double)s + (double)lo : (double)s; }
 };
 
 template <typename XT, typename GT>
@@ -415,7 +418,7 @@ __global__ void __launch_bounds__(kElemThreads, kMomCtas)
     const GT* src = static_cast<const GT*>(MODE == 0 ? grads[d.grad_slot] : d.w);
     const SquareSum acc = momentum_chunk<XT>(d, ch.begin, ch.count, src, k, MODE);
     // ||G_hat||_F^2: warp shuffle and shared memory, one fp64 atomic per chunk
-    double sum = (double)acc.s + (double)acc.lo;
+    double sum = acc.total();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;

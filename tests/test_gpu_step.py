@@ -403,3 +403,29 @@ def test_nonfinite_matrix_leaves_the_others_alone(env, cfg, monkeypatch):
         opt.close()
     for a, b in zip(*runs):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(64, 96), (33, 301), (5, 3)])   # whole vectors in a row, ragged rows, less than a vector
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_norm_overflow_without_iterations(shape, dtype):
+    """Finite entries whose squares overflow fp32, ns_steps = 0: the norm is
+    infinite (LM_FLAG_NONFINITE) and X / (norm + eps) zero, so a Muon step
+    only decays the parameter and an msign is zero; a NaN from the norm would
+    reach every entry."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    x = host_tensor(synth.draw_matrix(shape, seed=3) * 1e22, dtype).cuda()
+    assert bool(torch.isfinite(x.float()).all())
+    out = torch.full(shape, 7.0, device="cuda")
+    L.msign_ns(x, out, 0)
+    assert not out.any()
+    w0 = host_tensor(synth.init_weights([shape], seed=2)[0], dtype)
+    p = w0.cuda()
+    opt = L.LionMuon([p], period=1, eta_muon=0.1, weight_decay=0.5, ns_steps=0)
+    opt.step([x], 0)
+    torch.cuda.synchronize()
+    assert opt.status() == L.LM_FLAG_NONFINITE
+    opt.close()
+    w = w0.float().numpy()
+    want = w - np.float32(0.1) * (np.float32(0.5) * w)   # each operation rounded, as the kernels do
+    np.testing.assert_array_equal(bits(p), bits(host_tensor(want, dtype)))
