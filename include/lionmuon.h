@@ -238,6 +238,11 @@ lm_status lm_create(const lm_tensor* params, int n, const lm_config* cfg,
  * a graph of step k (0 <= k < period) serves every later step t with
  * t % period == k; the AdamW rule for vectors uses t itself (bias
  * correction).
+ * The tensor-core Newton-Schulz launches of a Muon step are cooperative and
+ * need their SMs (up to all of them) at the same time: a kernel of another
+ * stream that holds some delays them until it ends, so such a kernel must not
+ * wait for the step.  On a stream of a green context, which may have fewer SMs,
+ * they run phase by phase without that need (slower, same results).
  * After a captured step every later lm_step re-uploads its gradient pointers.
  * Replays and lm_step calls on one state must not overlap on the GPU.
  * Errors: LM_ERR_INVALID_ARG (n mismatch, t < 0, shape mismatch, NULL),

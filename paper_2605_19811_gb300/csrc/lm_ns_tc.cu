@@ -1582,18 +1582,34 @@ static cudaError_t set_smem_attr() {
                               (int)TcLayout<kP, kBN>::kSmemBytes);
 }
 
+// Whether launches on st run on a part of the device's SMs only (a stream of a
+// green context; a stream that cannot be asked is taken for one).
+static bool part_of_device(cudaStream_t st) {
+  static const PFN_cuStreamGetCtx_v12050 get = []() -> PFN_cuStreamGetCtx_v12050 {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &f, 12050, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<PFN_cuStreamGetCtx_v12050>(f);
+    return nullptr;
+  }();
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  return get == nullptr || get(st, &ctx, &green) != CUDA_SUCCESS || green != nullptr;
+}
+
 template <bool kSplit, int kP, int kBN, bool kPromo = false>
-static cudaError_t launch_chain(const ChainParams& prm, int grid, cudaStream_t st) {
+static cudaError_t launch_chain(const ChainParams& prm, int grid, bool together, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kChainThreads, 1, 1);
   cfg.dynamicSmemBytes = TcLayout<kP, kBN>::kSmemBytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;   // pairs wait for one another: all resident or none
+  attr[0].id = cudaLaunchAttributeCooperative;   // (together) pairs wait for one another: all resident or none
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = together ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, ns_tc_kernel<kSplit, kP, kBN, kPromo>, prm);
 }
 
@@ -1605,6 +1621,8 @@ int tc_max_pairs() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int pairs = sms / 2 > 0 ? sms / 2 : 1;
+  // (planned for the whole device, also from within a part of it)
+  if (sms > 0 && part_of_device(nullptr)) return pairs;
   // the pairs of a chain launch must all be resident at once
   if (set_smem_attr<true, 1, 256>() == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
@@ -1619,7 +1637,10 @@ int tc_max_pairs() {
   return pairs;
 }
 
-cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
+// What a launch runs of its phases: tiles and the sums of split Gram targets,
+// or one of the two.
+enum ChainPart { kTilesAndSums, kTilesOnly, kSumsOnly };
+static cudaError_t launch_chain_part(const NsChain& c, int q0, int q1, ChainPart part, bool together, cudaStream_t st) {
   if (q0 >= q1) return cudaSuccess;
   if (c.ngroups < 1 || c.ngroups > kMaxGroupsTc || c.steps < 1 || c.steps > kMaxNsSteps || c.npairs < 1 ||
       (c.pieces != 1 && c.pieces != 3) || (c.pieces == 3 && c.fuse != nullptr) || c.wait_ns == 0 ||
@@ -1680,8 +1701,8 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
   const bool global_w = last_fused && !(prm.it[c.steps - 1].mode & kIterFold);
   if (global_w && c.bn != 256) return cudaErrorInvalidValue;
   if (global_w && q0 != 3 * c.steps - 1) {
-    cudaError_t e = launch_ns_chain(c, q0, q1 - 1, st);
-    return e == cudaSuccess ? launch_ns_chain(c, q1 - 1, q1, st) : e;
+    cudaError_t e = launch_chain_part(c, q0, q1 - 1, part, together, st);
+    return e == cudaSuccess ? launch_chain_part(c, q1 - 1, q1, part, together, st) : e;
   }
   if (last_fused) prm.fuse = *c.fuse;
   const int base_epi = c.pieces == 3 && c.promote ? kEpiWarps : 4;
@@ -1692,16 +1713,43 @@ cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
   const int warps = 2 * c.npairs * kEpiWarps;
   prm.fin_units = 8;
   while (prm.fin_units < 64 && prm.fin_units * c.ntargets * 2 <= warps) prm.fin_units *= 2;
+  if (part == kTilesOnly) prm.ntargets = 0;
+  for (int ph = 0; ph < 3 && part == kSumsOnly; ++ph) {
+    prm.offsets[ph] = nullptr;
+    prm.ntiles[ph] = 0;
+    prm.counts = nullptr;
+  }
   const int grid = 2 * c.npairs;
   const bool split = c.ntargets > 0;
   count_launch();
   if (c.pieces == 3 && c.promote)
-    return split ? launch_chain<true, 3, 128, true>(prm, grid, st) : launch_chain<false, 3, 128, true>(prm, grid, st);
+    return split ? launch_chain<true, 3, 128, true>(prm, grid, together, st)
+                 : launch_chain<false, 3, 128, true>(prm, grid, together, st);
   if (c.pieces == 3)
-    return split ? launch_chain<true, 3, 128>(prm, grid, st) : launch_chain<false, 3, 128>(prm, grid, st);
+    return split ? launch_chain<true, 3, 128>(prm, grid, together, st)
+                 : launch_chain<false, 3, 128>(prm, grid, together, st);
   if (c.bn == 128)
-    return split ? launch_chain<true, 1, 128>(prm, grid, st) : launch_chain<false, 1, 128>(prm, grid, st);
-  return split ? launch_chain<true, 1, 256>(prm, grid, st) : launch_chain<false, 1, 256>(prm, grid, st);
+    return split ? launch_chain<true, 1, 128>(prm, grid, together, st)
+                 : launch_chain<false, 1, 128>(prm, grid, together, st);
+  return split ? launch_chain<true, 1, 256>(prm, grid, together, st)
+               : launch_chain<false, 1, 256>(prm, grid, together, st);
+}
+
+// On a part of the device the planned pairs may not all be resident, and no
+// launch may wait for another pair: one launch per phase, and one more for the
+// sums of a phase's split Gram targets, neither cooperative (a cooperative
+// launch larger than the part does not return).  Then every counter a launch
+// waits for was reached by the launches before it.
+cudaError_t launch_ns_chain(const NsChain& c, int q0, int q1, cudaStream_t st) {
+  if (!part_of_device(st)) return launch_chain_part(c, q0, q1, kTilesAndSums, true, st);
+  for (int q = q0; q < q1; ++q) {
+    if (q % 3 == NS_POLY && ns_iter_form(c.co[q / 3], c.pieces, c.fold).from_a) continue;
+    cudaError_t e = launch_chain_part(c, q, q + 1, kTilesOnly, false, st);
+    if (e == cudaSuccess && q % 3 == NS_GRAM && c.ntargets > 0)
+      e = launch_chain_part(c, q, q + 1, kSumsOnly, false, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_ns_wide_phase(NsPhase ph, int iter, int ngroups, const NsGroup* groups, const TcGroupMaps* maps,

@@ -194,3 +194,83 @@ def test_vectors_in_the_momentum_launch(n, dtype):
         got.append([bits(p) for p in params] + [bits(opt.momentum(i)) for i in range(3)])
     for x, y in zip(*got):
         np.testing.assert_array_equal(x, y)
+
+
+# ------------------------- beside other work -------------------------------
+def test_step_beside_another_streams_kernel():
+    """The chain needs its SMs at the same time; a kernel of another stream
+    that holds one delays it and changes nothing."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    shapes = [(768, 768), (768, 3072), (3072, 768)]
+    grads = [host_tensor(x, "bf16").cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=0)]
+    got = []
+    for busy in (False, True):
+        params = [host_tensor(w, "bf16").cuda() for w in synth.init_weights(shapes, seed=1)]
+        opt = L.LionMuon(params, period=1)
+        other = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        for t in range(3):
+            if busy:
+                with torch.cuda.stream(other):
+                    torch.cuda._sleep(2_000_000)   # about a millisecond on one SM
+            opt.step(grads, t)
+        torch.cuda.synchronize()
+        assert opt.status() == 0
+        got.append([bits(p) for p in params])
+        opt.close()
+    for x, y in zip(*got):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.fixture
+def green_stream():
+    """A stream on 32 of the device's SMs (a green context)."""
+    import ctypes
+    import torch
+    torch.zeros(1, device="cuda")
+    cu = ctypes.CDLL("libcuda.so.1")
+    res, part, rest = (ctypes.create_string_buffer(256) for _ in range(3))   # CUdevResource is 144 bytes
+    n, desc, ctx, stream = ctypes.c_uint(1), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    sm = 1                                                                   # CU_DEV_RESOURCE_TYPE_SM
+    if (cu.cuDeviceGetDevResource(0, res, sm) or cu.cuDevSmResourceSplitByCount(part, ctypes.byref(n), res, rest, 0, 32)
+            or cu.cuDevResourceGenerateDesc(ctypes.byref(desc), part, 1)
+            or cu.cuGreenCtxCreate(ctypes.byref(ctx), desc, 0, 1) or cu.cuGreenCtxStreamCreate(ctypes.byref(stream), ctx, 1, 0)):
+        pytest.skip("no green contexts")
+    yield torch.cuda.ExternalStream(stream.value)
+    assert cu.cuStreamSynchronize(stream) == 0
+    cu.cuStreamDestroy_v2(stream)
+    cu.cuGreenCtxDestroy(ctx)
+
+
+@pytest.mark.parametrize("precision,dtype,shapes,cfg", [
+    (1, "bf16", [(768, 768), (20000, 768), (768, 2304), (768,)], {}),    # Gram tiles split along K
+    (1, "bf16", [(512, 1024), (1024, 512)] * 3, dict(schedule=1, srank_alpha=0.02)),
+    (1, "bf16", [(512, 640), (640, 512)], dict(ns_coeffs=((4.1, -3.1, 0.6), (1.5, -0.5, 0.0)))),   # a cubic last
+    (2, "f32", [(768, 768), (20000, 768)], {}),
+    (0, "f32", [(1024, 1024), (1100, 9000)], {})])
+def test_part_of_the_device(precision, dtype, shapes, cfg, green_stream):
+    """Steps on a stream that has fewer SMs than the state was planned for run
+    there (a launch per phase, none of which waits for another pair), with the
+    same results; the static-area msign too."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    cfg = dict(period=1, **cfg) if "schedule" not in cfg else cfg
+    grads = [[host_tensor(x, dtype).cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=t)] for t in range(2)]
+    got = []
+    for stream in (None, green_stream):
+        params = [host_tensor(w, dtype).cuda() for w in synth.init_weights(shapes, seed=1)]
+        x = host_tensor(synth.draw_matrix((768, 2048), seed=3), "bf16").cuda()
+        out = torch.empty((768, 2048), device="cuda")
+        torch.cuda.synchronize()
+        opt = L.LionMuon(params, stream=stream, ns_precision=precision, **cfg)
+        for t in range(2):
+            opt.step(grads[t], t, stream=stream)
+        L.msign_ns_noalloc(x, out, stream=stream)
+        assert L.msign_ns_noalloc_status(stream=stream) == (0, 0)
+        assert opt.status() == 0
+        torch.cuda.synchronize()
+        got.append([bits(p) for p in params] + [bits(opt.momentum(i)) for i in range(len(params))] + [bits(out)])
+        opt.close()
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
