@@ -270,6 +270,7 @@ int sm_count() {
 // accumulator.  Measured on a 720M-set Muon step: the largest direction error
 // 2.5e-5 at 96 blocks, 1.2e-5 at 48, 8.8e-6 at 32, 8.4e-6 at 24.
 constexpr int kGramCapF32TC = 24;
+constexpr int64_t kMaxPartBlocks = 65535;   // split-K parts of a batch, in 256 x 256 blocks (256 KB of fp32 each)
 constexpr int kMaskedGramPart = 200;   // longest Gram part of a large masked batch (K blocks)
 // K blocks that cutting a Gram tile has to save in a small batch: writing the
 // parts, waiting for them and summing them takes about 7 us more than writing a
@@ -507,7 +508,7 @@ struct NsLayout {
 // long-K embedding Gram next to short hidden matrices, which would otherwise
 // set the length of the launch - is cut into parts of at most half that load.
 // Each part is a tile of its own for the scheduler and writes its partial
-// product to a workspace tile of its own (slot = part index + 1); the finish
+// product to a workspace tile of its own (tc_part); the finish
 // kernel adds the parts in order, so the result does not depend on timing.
 // Tiles near the average stay whole: splitting them buys no balance.
 // kcap > 0 also splits every tile longer than kcap K slices into parts of at
@@ -554,15 +555,23 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
     keep = std::min<int64_t>(keep, kMaskedGramPart);
     part = std::min<int64_t>(part, kMaskedGramPart);
   }
-  if (kcap > 0) part = std::min<int64_t>(part, kcap);
+  // The parts' workspace: at most kMaxPartBlocks blocks.  Where kcap asks for
+  // more (15 layers of d = 4096, say), the shortest cap that fits bounds every
+  // tile, so that none is left whole.
+  const int64_t want = part;
   std::vector<char> whole(ng, 0);
-  int64_t planned = 0;   // part numbers are 16 bits (a block may be two tiles wide)
-  for (int g = 0; g < ng; ++g) {
-    const int64_t n = 2 * blocks[g] * std::min<int64_t>(64, (len[g] + part - 1) / part);
-    whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || planned + n > 65535 ||
-               (kcap <= 0 && avg < 32 && len[g] - part < worth);
-    if (!whole[g]) planned += n;
-  }
+  int64_t planned;
+  do {
+    if (kcap > 0) part = std::min<int64_t>(want, kcap);
+    planned = 0;
+    for (int g = 0; g < ng; ++g) {
+      const int64_t n = blocks[g] * std::min<int64_t>(64, (len[g] + part - 1) / part);
+      whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || (kcap <= 0 && planned + n > kMaxPartBlocks) ||
+                 (kcap <= 0 && avg < 32 && len[g] - part < worth);
+      if (!whole[g]) planned += n;
+    }
+    kcap += kcap > 0 ? 1 : 0;
+  } while (planned > kMaxPartBlocks && kcap <= longest);
   std::vector<NsTile> out;
   nparts_total = 0;
   for (const NsTile& x0 : t) {
@@ -583,7 +592,8 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
         NsTile y = x;
         y.kb0 = (uint16_t)(nk * k / nparts);
         y.kb1 = (uint16_t)(nk * (k + 1) / nparts);
-        y.slot = (uint16_t)(nparts_total + k + 1);
+        y.slot = (uint16_t)((nparts_total + k) % kPartsPerSlotWrap + 1);
+        y.nh = (uint16_t)((nparts_total + k) / kPartsPerSlotWrap);
         out.push_back(y);
       }
       nparts_total += nparts;

@@ -174,10 +174,15 @@ struct alignas(16) NsTile {
   // written in fp32 to workspace tile slot - 1, and the parts are summed.
   uint16_t kb0, kb1, slot;
   // 256-column output blocks of the tile, starting at block tn: 2 only in
-  // the wide-tile kernel's launches (0 and 1 both mean one block); the fp32
-  // path's split tiles: part index << 8 | parts.
+  // the wide-tile kernel's launches (0 and 1 both mean one block); split
+  // tiles: of the fp32 path part index << 8 | parts, of the chain kernel the
+  // upper half of the part's number (tc_part).
   uint16_t nh;
 };
+// Workspace tile of a split-K part on the tensor-core path, whose part numbers
+// pass 16 bits for large three-piece sets: slot stays 1 .. 65535.
+constexpr int kPartsPerSlotWrap = 65535;
+inline __host__ __device__ int tc_part(const NsTile& t) { return (int)t.nh * kPartsPerSlotWrap + (int)t.slot - 1; }
 // A split Gram tile of the tensor-core path (256 rows, 256 or 128 columns): the
 // parts in workspace tiles first .. first + nparts - 1 are summed in that
 // order (so the result does not depend on timing) and written to A at

@@ -196,6 +196,28 @@ def test_vectors_in_the_momentum_launch(n, dtype):
         np.testing.assert_array_equal(x, y)
 
 
+def test_three_piece_gram_parts_of_a_large_matrix():
+    """A matrix whose Gram tiles come to more than 65535 parts of 128 columns
+    (20480 x 20480: 3240 blocks of 256 x 256, 14 parts each) keeps the bound on
+    the length of a sum in tensor-core accumulators (24 K blocks).  A A^T X
+    alone (one iteration, (a, b, c) = (0, 1, 0)) on some columns against fp64:
+    the products of K = 20480 of APPLY, which are not cut, leave 2.5e-5; with
+    whole Gram tiles (320 K blocks) it was 7.6e-5."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    n = 20480
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(2)
+    x = torch.randn((n, n), generator=gen, device="cuda")
+    out = torch.empty_like(x)
+    L.msign_ns(x, out, 1, 0.0, 1.0, 0.0, precision=L.LM_NS_F32_TC)
+    rows = [x[i:i + 2048] for i in range(0, n, 2048)]
+    v = sum(r.double().t() @ r[:, :64].double() for r in rows)
+    norm = sum(float(r.double().square().sum()) for r in rows) ** 0.5
+    want = torch.cat([r.double() @ v for r in rows]) / (norm + 1e-7) ** 3
+    assert float((out[:, :64].double() - want).norm() / want.norm()) <= 4e-5
+
+
 # ------------------------- beside other work -------------------------------
 def test_step_beside_another_streams_kernel():
     """The chain needs its SMs at the same time; a kernel of another stream
