@@ -283,10 +283,12 @@ lm_status lm_set_second_moment(lm_state* s, int i, const lm_tensor* src,
  * coefficients (a, b, c), normalisation X / (||X||_F + eps), iterated on the
  * wide orientation, with no 0.2 sqrt(max(m,n)) scaling.  in and out are
  * device tensors of equal shape (rows, cols >= 2 each), dtype LM_BF16 or
- * LM_F32 (may differ).  precision as lm_config::ns_precision.  Allocates its workspace with stream-ordered
- * allocation on cuda_stream and frees it the same way.  A testing entry
- * point: it synchronises cuda_stream before it returns, to read its own
- * status word.
+ * LM_F32 (may differ).  precision as lm_config::ns_precision.  Allocates its
+ * workspace with stream-ordered allocation on cuda_stream and frees it the
+ * same way.  A testing entry point: it synchronises cuda_stream before it
+ * returns, to read its own status word.  A workspace above 256 MiB is back
+ * with the device by then; a smaller one stays in the device's default memory
+ * pool until the program next synchronises.
  * Errors: LM_ERR_INVALID_ARG, LM_ERR_DTYPE, LM_ERR_ALIGN, LM_ERR_OOM,
  * LM_ERR_CUDA, LM_ERR_TIMEOUT (a bounded device wait gave up; the kernels
  * after it did nothing and out holds no result). */

@@ -288,6 +288,12 @@ constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
 // launch, 7370 per phase.  Below, one launch wins: 355M-shaped set (2600) 4.83 ms
 // per Muon step against 5.00, 124M-shaped 1515 us against 1672.
 constexpr int kPhaseLaunchBlocks = 4096;
+// Largest msign workspace that stays in the stream-ordered pool until the
+// program's next synchronisation: 0.1% of the device, so that a caller's own
+// allocation after the call does not miss it.  Past it the memory's return and
+// renewal cost 0.5 ms (4096 x 4096 bf16, 1.0 ms) to 3.5 ms a call (50304 x 2048
+// fp32, 14.9 ms).
+constexpr size_t kMsignKeepBytes = (size_t)256 << 20;
 constexpr uint64_t kRingWaitNs = 2000000000ull;   // the power-iteration ring's waits: 2 s unless set shorter
 
 struct LionTable {
@@ -2159,7 +2165,8 @@ static lm_status msign_run(const lm_tensor* in, lm_tensor* out, int steps, const
 
   const size_t off_tab = align_up(buf.total, 256);
   char* mem = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&mem), off_tab + ar.total, stream);
+  const size_t total = off_tab + ar.total;
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&mem), total, stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(msign workspace)");
   char* base = mem + off_tab;
   std::vector<char> img(ar.total, 0);
@@ -2204,14 +2211,17 @@ static lm_status msign_run(const lm_tensor* in, lm_tensor* out, int steps, const
   if ((st = run_ns(E, steps, co.data(), dflags, stream)) != LM_OK) return cleanup(st);
   e = launch_finalize(xio, out->dtype, dm, de, (int)et.size(), mk, 1, dflags, stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "output kernel launch"));
-  // The call's status word, read back before the workspace goes.  The
-  // workspace is freed after the synchronisation: the stream-ordered pool then
-  // still has it for a call that follows, and gives it back to the device at
-  // the program's next synchronisation.
+  // The call's status word, read back before the workspace goes.  A workspace
+  // freed before the synchronisation returns to the device with it; freed
+  // after it, the stream-ordered pool still has it for a call that follows, and
+  // gives it back at the program's next synchronisation (msign of 1280 x 5120:
+  // 366 us a call against 633).  Only a small one stays in the pool.
+  const bool keep = total <= kMsignKeepBytes;
   unsigned hflags = 0;
   e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, stream);
+  if (!keep) cudaFreeAsync(mem, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  cudaFreeAsync(mem, stream);
+  if (keep) cudaFreeAsync(mem, stream);
   if (e != cudaSuccess) return cuda_fail(e, "msign status read");
   if (hflags & LM_FLAG_TIMEOUT)
     return fail(LM_ERR_TIMEOUT, "a bounded device wait gave up; out was not written (LM_FLAG_TIMEOUT)");

@@ -205,3 +205,18 @@ def test_msign_three_piece_mode_not_in_noalloc_entry():
     with pytest.raises(L.LionMuonError) as e:
         L.msign_ns_noalloc(x, out, 5, *QUINTIC, precision=L.LM_NS_F32_TC)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("shape,precision", [((50304, 1024), 0), ((8192, 8192), 1)])
+def test_large_workspace_goes_back_to_the_device(shape, precision):
+    """A workspace above 256 MiB does not stay in the memory pool when the call
+    returns: the caller's next cudaMalloc can have it."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    x = torch.randn(shape, device="cuda")
+    out = torch.empty_like(x)
+    L.msign_ns(x[:64], out[:64], precision=precision)   # the library and the pool are up
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    L.msign_ns(x, out, precision=precision)
+    assert before - torch.cuda.mem_get_info()[0] <= 256 << 20
