@@ -112,10 +112,12 @@ typedef struct {
  * three bf16 pieces hi + mid + lo and a product sums the six piece products
  * down to order 2^-16, accumulated in fp32; the fast fp32 mode, at the cost of
  * six bf16 products per product) or LM_F32 (the exact fp32 mode: fp32 FMA on
- * the CUDA cores, or, where every matrix has at least 320 rows and columns (256
- * when every |a_k| < 4) and the workspace fits, the three pieces with their
- * main products summed in fp32 registers per 64-deep block, which is closer to
- * the fp64 iteration than the FMAs).
+ * the CUDA cores, or, where every matrix is wide enough and the workspace fits,
+ * the three pieces with their main products summed in fp32 registers per
+ * 64-deep block, which is at least as close to the fp64 iteration as the FMAs
+ * there: at least 512 rows and columns, 1024 for more than 5 iterations, 256
+ * for up to 5 of the default quintic on a matrix at most four times as long as
+ * wide).
  * ns_coeffs: NULL for the same (ns_a, ns_b, ns_c) in every NS iteration, or
  * 3 * ns_steps finite values (a_k, b_k, c_k), k = 0 .. ns_steps - 1, for
  * iteration-dependent odd polynomials X <- a_k X + (b_k A + c_k A^2) X, the

@@ -929,21 +929,30 @@ static cudaError_t timed(Profiler* P, int fam, cudaStream_t st, F&& f) {
 
 // Where full-fp32 Newton-Schulz (LM_F32) runs on the tensor cores as three bf16
 // pieces with the main products summed in registers (NsChain::promote): for
-// sets all of whose matrices are wide enough that this is closer to the fp64
-// iteration than fp32 FMAs are.  Measured over 8 to 20000 rows and columns, four
-// kinds of input, each against fp64: from 333 up it is 0.15 to 0.8 times as
-// far with the quintic and the degree-5 minimax table, at 256 0.26 to 0.63
-// with the quintic but up to 1.2 with the table (whose first |a| is 8.5);
-// narrower matrices go either way (130 x 200: 0.37 to 6).  An msign of 1024 x
-// 1024 takes 465 us there against 1026 us, a step of the 124M-shaped set (P = 2)
-// 5.1 ms against 17.4.
+// sets all of whose matrices are wide enough that this is no further from the
+// fp64 iteration than fp32 FMAs are.  The FMAs' error grows with the width and
+// is random; the tensor cores' is smaller but leans one way (sums truncate), so
+// what the iteration amplifies, long products and many steps, counts against
+// them.  Mean distance from fp64 over that of the FMAs, s = 256 .. 1280, l = s ..
+// 50304, normal and Student-t inputs (s the smaller side):
+//   default quintic, up to 5 steps   0.21-0.97 from s = 512, and from 256 where
+//                                    l <= 4 s; past that 320-480 reach 1.4
+//   other tables of up to 5 steps    0.22-0.81 from 512 (degree-5 minimax,
+//                                    1.875/-1.25/0.375, cubic); 320-384 1.4
+//   10 steps of the quintic          0.25-0.77 from 1024; 512-768 1.6
+// An msign of 1024 x 1024 takes 465 us there against 1026 us, a step of the
+// 124M-shaped set (P = 2) 5.1 ms against 17.4.
 static bool f32_on_tensor_cores(const std::vector<std::pair<int64_t, int64_t>>& shapes, const std::vector<NsCoeffs>& co) {
-  int64_t least = 320;
-  bool small_a = true;
-  for (const NsCoeffs& c : co) small_a = small_a && std::fabs(c.a) < 4.f;
-  if (small_a) least = 256;
-  for (const auto& x : shapes)
-    if (std::min(x.first, x.second) < least) return false;
+  lm_config def;
+  lm_config_default(&def);
+  bool quintic = co.size() <= 5;
+  for (const NsCoeffs& c : co)
+    quintic = quintic && c.a == (float)def.ns_a && c.b == (float)def.ns_b && c.c == (float)def.ns_c;
+  for (const auto& x : shapes) {
+    const int64_t s = std::min(x.first, x.second), l = std::max(x.first, x.second);
+    const int64_t least = quintic && l <= 4 * s ? 256 : (co.size() <= 5 ? 512 : 1024);
+    if (s < least) return false;
+  }
   return !shapes.empty() && !co.empty();
 }
 

@@ -120,11 +120,13 @@ def test_ragged_rows_step(shape, dtype, precision):
     opt.close()
 
 
-# Full-fp32 mode around the choice of its path (256 rows with the quintic, 320
-# with a table whose |a| reaches 8.5), and on the CUDA cores: one 64-wide tile
-# and just past it, tiles cut along K, 128-wide tiles
+# Full-fp32 mode around the choice of its path (with the quintic 256 rows, 512
+# where the matrix is more than four times as long; 512 with another table),
+# and on the CUDA cores: one 64-wide tile and just past it, tiles cut along K,
+# 128-wide tiles
 @pytest.mark.parametrize("shape", [(255, 600), (256, 600), (600, 256), (319, 700), (700, 320), (2, 64), (65, 64),
-                                   (64, 5000), (250, 9000), (1000, 1024)])
+                                   (64, 5000), (250, 9000), (1000, 1024), (256, 1024), (1025, 256), (511, 2100),
+                                   (2100, 512)])
 def test_full_fp32_msign(shape):
     import torch
     from paper_2605_19811_gb300 import lionmuon as L
@@ -194,6 +196,43 @@ def test_vectors_in_the_momentum_launch(n, dtype):
         got.append([bits(p) for p in params] + [bits(opt.momentum(i)) for i in range(3)])
     for x, y in zip(*got):
         np.testing.assert_array_equal(x, y)
+
+
+# long products, split along K, in the full-fp32 mode on either path
+@pytest.mark.parametrize("shape", [(320, 20000), (512, 20000), (20000, 555)])
+def test_full_fp32_msign_long(shape):
+    xh = host_tensor(synth.draw_matrix(shape, seed=shape[0]), "f32")
+    want = ns_closed_form_rows(stored_values(xh), 5, *QUINTIC, 1e-7)
+    assert rel_fro(tall(_msign(xh, 0)), want) <= 1e-5
+
+
+@pytest.mark.parametrize("shape,table", [((384, 15360), (QUINTIC,) * 5), ((480, 1440), (QUINTIC,) * 10),
+                                         ((336, 504), "polar"), ((512, 768), "polar"), ((256, 1024), (QUINTIC,) * 5),
+                                         ((1024, 1100), (QUINTIC,) * 10)])
+def test_full_fp32_is_as_close_as_the_cuda_cores(shape, table, monkeypatch):
+    """Whatever path LM_F32 takes, its direction is no further from fp64 than
+    the CUDA cores' (the path it falls back to without the workspace), 10%
+    allowed for the draw: the mean over inputs is below 1 where it takes the
+    other one, 1.26 to 1.4 in the first three cases if it did."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    from paper_2605_19811_gb300.ns_coeffs import polar_express
+    table = polar_express(5) if table == "polar" else table
+    err = []
+    x = host_tensor(synth.draw_matrix(shape, seed=shape[1]), "f32")
+    want = O.ns_polynomial_schedule(stored_values(x), table, 1e-7)
+    for fault in (None, "oom_f32tc"):
+        if fault:
+            monkeypatch.setenv("LM_FAULT", fault)
+        w = torch.zeros(shape, device="cuda")
+        opt = L.LionMuon([w], period=1, eta_muon=1.0, weight_decay=0.0, beta1=0.0, shape_scale=1.0, ns_precision=0,
+                         ns_coeffs=table)
+        opt.step([x.cuda()], 0)   # W = -sqrt(max(m, n)) NS(G)
+        torch.cuda.synchronize()
+        assert opt.status() == 0
+        err.append(rel_fro(-stored_values(w) / max(shape) ** 0.5, want))
+        opt.close()
+    assert err[0] <= 1.1 * err[1], err
 
 
 def test_three_piece_gram_parts_of_a_large_matrix():
