@@ -617,10 +617,7 @@ def run_ours(args):
     pk_bf16 = pk_sust if long_region else pk_burst
     bf16_kind = (f"bf16 {'sustained' if long_region else 'burst'} ({ms_total / 1e3:.2f} s timed region), "
                  f"{peak_src}")
-    # fp32 modes on the tensor cores: LM_NS_F32_TC, and LM_F32 where every matrix
-    # is wide enough (256 where all |a| < 4, 320 otherwise)
-    least = 256 if table is None or all(abs(row[0]) < 4 for row in table) else 320
-    pieces = args.precision == "f32tc" or (args.precision == "f32" and min(min(m) for m in ns_mats) >= least)
+    pieces = opt.ns_path() == L.LM_NS_F32_TC   # fp32 on the tensor cores (LM_NS_F32_TC, or LM_F32 where it takes them)
     roof = None
     if ns_ms > 0 and n_muon > 0:
         achieved = fl / (ns_ms / 1e3) / 1e12

@@ -369,6 +369,15 @@ size_t lm_state_bytes(const lm_state* s);
  * buffers, tables).  Returns 0 for NULL. */
 size_t lm_workspace_bytes(const lm_state* s);
 
+/* What the state's Newton-Schulz products run on: LM_BF16 (bf16 operands on the
+ * tensor cores), LM_NS_F32_TC (fp32 operands as three bf16 pieces on the tensor
+ * cores) or LM_F32 (fp32 FMA on the CUDA cores).  A state with ns_precision
+ * LM_F32 takes one of the last two when it is created, by its shapes and
+ * coefficients and by whether the larger workspace of the pieces (16 bytes per
+ * element of X and 12 per element of A and B, against 8 and 8) fits the device;
+ * their results differ in the last bits.  Returns -1 for NULL. */
+int lm_ns_path(const lm_state* s);
+
 /* Synchronise the state's last stream and free everything it owns.  NULL is
  * a no-op. */
 void lm_destroy(lm_state* s);

@@ -2117,6 +2117,11 @@ size_t lm_workspace_bytes(const lm_state* s) {
   return s ? s->bytes - (s->mom_elems + s->v_elems) * sizeof(float) : 0;
 }
 
+int lm_ns_path(const lm_state* s) {
+  if (s == nullptr) return -1;
+  return s->ns.xdt == LM_F32 ? LM_F32 : (s->ns.pieces == 3 ? LM_NS_F32_TC : LM_BF16);
+}
+
 void lm_destroy(lm_state* s) {
   if (s == nullptr) return;
   cudaStreamSynchronize(s->last_stream);

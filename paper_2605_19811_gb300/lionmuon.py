@@ -31,7 +31,7 @@ EXPORTED = ("lm_config_default", "lm_create", "lm_step", "lm_set_lr", "lm_msign_
             "lm_kernel_launch_count", "lm_profile_enable", "lm_profile_read",
             "lm_msign_ns_noalloc", "lm_probe_bounded_wait", "lm_msign_ns_coeffs",
             "lm_set_adamw_lr", "lm_get_second_moment", "lm_set_second_moment", "lm_get_selection",
-            "lm_msign_ns_noalloc_status", "lm_shard_owners", "lm_config_size")
+            "lm_msign_ns_noalloc_status", "lm_shard_owners", "lm_config_size", "lm_ns_path")
 
 KERNEL_FAMILIES = ("lion", "momentum_norm", "ns_gram", "ns_poly", "ns_apply", "finalize", "other", "adamw",
                    "srank")
@@ -128,6 +128,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.lm_state_bytes.restype = ctypes.c_size_t
     lib.lm_workspace_bytes.argtypes = [c_void_p]
     lib.lm_workspace_bytes.restype = ctypes.c_size_t
+    lib.lm_ns_path.argtypes = [c_void_p]
+    lib.lm_ns_path.restype = c_int
     lib.lm_destroy.argtypes = [c_void_p]
     lib.lm_destroy.restype = None
     lib.lm_status_string.argtypes = [c_int]
@@ -333,6 +335,11 @@ class LionMuon:
 
     def workspace_bytes(self) -> int:
         return int(self._lib.lm_workspace_bytes(self._h))
+
+    def ns_path(self) -> int:
+        """What the Newton-Schulz products run on: LM_BF16, LM_NS_F32_TC (three
+        bf16 pieces on the tensor cores) or LM_F32 (CUDA cores)."""
+        return int(self._lib.lm_ns_path(self._h))
 
     def close(self) -> None:
         if getattr(self, "_h", None):

@@ -165,6 +165,7 @@ def test_full_fp32_falls_back_without_the_workspace(monkeypatch):
         opt.step(g, 0)
         torch.cuda.synchronize()
         assert opt.status() == 0
+        assert opt.ns_path() == (L.LM_F32 if fault else L.LM_NS_F32_TC)
         out.append(([stored_values(p) for p in params], opt.workspace_bytes()))
         opt.close()
     assert out[1][1] != out[0][1]
