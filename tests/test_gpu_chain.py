@@ -45,6 +45,8 @@ def _steps(shapes, profile, steps=3, dtype="bf16", **cfg):
     from paper_2605_19811_gb300 import lionmuon as L
     params = [host_tensor(w, dtype).cuda() for w in synth.init_weights(shapes, seed=1)]
     opt = L.LionMuon(params, **cfg)
+    if dtype == "f32" and cfg["ns_precision"] == 0:
+        assert opt.ns_path() == L.LM_NS_F32_TC
     opt.profile(profile)
     for t in range(steps):
         opt.step([host_tensor(x, dtype).cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=t)], t)
@@ -65,8 +67,17 @@ CASES = [(NINE, {}), ([(768, 768), (20000, 768), (768, 2304), (768,)], {}),
          ([(512, 1024), (1024, 512)] * 3, dict(schedule=1, srank_alpha=0.02))]
 
 
-@pytest.mark.parametrize("shapes,cfg", CASES)
-@pytest.mark.parametrize("precision,dtype", [(1, "bf16"), (2, "f32")])
+# the same kinds for the full-fp32 mode with register sums (every matrix wide
+# enough for it): nine shapes, a long Gram split along K next to short matrices,
+# tables with and without a cubic, the mask
+WIDE_CASES = [([(320 + 32 * k, 448 + 32 * k) for k in range(9)], {}),
+              ([(768, 768), (20000, 768), (768, 2304), (768,)], {}),
+              ([(512, 640), (640, 512)], dict(ns_coeffs=((8.4, -25.0, 18.0), (4.1, -3.1, 0.6), (1.5, -0.5, 0.0)))),
+              ([(512, 1024), (1024, 512)] * 3, dict(schedule=1, srank_alpha=0.02))]
+
+
+@pytest.mark.parametrize("precision,dtype,shapes,cfg", [(p, d, *c) for p, d in ((1, "bf16"), (2, "f32")) for c in CASES] +
+                         [(0, "f32", *c) for c in WIDE_CASES])
 def test_one_launch_equals_one_launch_per_phase(shapes, cfg, precision, dtype):
     """With profiling on every phase has a launch of its own: the same tiles
     without the overlap of phases, so a missing dependency would show."""
@@ -199,6 +210,63 @@ def test_vectors_in_the_momentum_launch(n, dtype):
         np.testing.assert_array_equal(x, y)
 
 
+def _device_step(shapes, profile, ranked=(), steps=1, **cfg):
+    """Steps over bf16 sets too large to draw on the host; the matrices in
+    ``ranked`` have a dominant direction in their gradients.  Returns the bits,
+    the selection of the last step and its kernel launches."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+
+    def rand(s):
+        return torch.randn(s, generator=gen, device="cuda")
+    params = [(rand(s) * 0.02).bfloat16() for s in shapes]
+    grads = [rand(s) for s in shapes]
+    for i in ranked:
+        grads[i] += 0.5 * rand(shapes[i][:1])[:, None] * rand(shapes[i][1:])[None, :]
+    grads = [g.bfloat16() for g in grads]
+    opt = L.LionMuon(params, **cfg)
+    opt.profile(profile)
+    for t in range(steps):
+        n0 = L.kernel_launch_count()
+        opt.step(grads, t)
+        launches = L.kernel_launch_count() - n0
+    torch.cuda.synchronize()
+    assert opt.status() == 0
+    out = [bits(x) for i in range(len(shapes)) for x in (params[i], opt.momentum(i))]
+    took = opt.selection()[0]
+    opt.close()
+    return out, took, launches
+
+
+@pytest.mark.parametrize("shapes,ranked", [
+    ([(20000, 768), (768, 768), (768, 2304), (20000, 768)], (0, 1)),    # a light batch: Grams cut for the longest
+    ([(16384, 2048), (2048, 2048), (16384, 2048)], (2,))])              # a heavy one: parts capped under the mask
+def test_masked_lists_with_split_grams(shapes, ranked):
+    """Selected and skipped matrices, both with Gram tiles split along K: one
+    launch equals one launch per phase."""
+    cfg = dict(schedule=1, srank_alpha=0.03, steps=3, ranked=ranked)
+    a, took, _ = _device_step(shapes, False, **cfg)
+    b, _, _ = _device_step(shapes, True, **cfg)
+    assert took == [i in ranked for i in range(len(shapes))]
+    for x, y in zip(a, b):
+        np.testing.assert_array_equal(x, y)
+
+
+def test_launch_per_phase_by_size_equals_one_launch():
+    """A batch large enough for a launch per phase (nine 4096 x 4096: 4377 K
+    blocks per CTA pair and iteration, from 4096), against the same tiles in
+    one launch: under the stable-rank mask a batch always takes one, and at
+    alpha = 1 every matrix is selected."""
+    shapes = [(4096, 4096)] * 9
+    a, _, na = _device_step(shapes, False, period=1)
+    b, took, nb = _device_step(shapes, False, schedule=1, srank_alpha=1.0)
+    assert all(took) and na - nb > 0, (na, nb)
+    for x, y in zip(a, b):
+        np.testing.assert_array_equal(x, y)
+
+
 # long products, split along K, in the full-fp32 mode on either path
 @pytest.mark.parametrize("shape", [(320, 20000), (512, 20000), (20000, 555)])
 def test_full_fp32_msign_long(shape):
@@ -256,6 +324,44 @@ def test_three_piece_gram_parts_of_a_large_matrix():
     norm = sum(float(r.double().square().sum()) for r in rows) ** 0.5
     want = torch.cat([r.double() @ v for r in rows]) / (norm + 1e-7) ** 3
     assert float((out[:, :64].double() - want).norm() / want.norm()) <= 4e-5
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_fp32_chain_from_a_graph_and_sharded(precision):
+    """The fp32 modes replayed from a CUDA graph equal eager steps; two sharded
+    states, each with the tiles of its own matrices, give the single state's
+    parameters within the modes' error (Gram tiles are cut otherwise)."""
+    import torch
+    from paper_2605_19811_gb300 import lionmuon as L
+    from paper_2605_19811_gb300 import shard
+    shapes = [(512, 640), (1400, 512), (640, 512), (512, 1400)]
+    cfg = dict(period=1, eta_muon=0.02, ns_precision=precision)
+    grads = [host_tensor(x, "f32").cuda() for x in synth.draw_grads(shapes, "student_t", seed=0, step=0)]
+
+    def fresh(**kw):
+        p = [host_tensor(w, "f32").cuda() for w in synth.init_weights(shapes, seed=1)]
+        return p, L.LionMuon(p, **cfg, **kw)
+    eager, opt = fresh()
+    replayed, graphed = fresh()
+    graph = graphed.capture_steps(grads)[0]
+    for t in range(2):
+        opt.step(grads, t)
+        graph.replay()
+    own = shard.owners(shapes, 2)
+    ranks = [fresh(shard_rank=r, shard_world=2) for r in range(2)]
+    for t in range(2):
+        for p, o in ranks:
+            o.step(grads, t)
+        for i, r in enumerate(own):
+            ranks[1 - r][0][i].copy_(ranks[r][0][i])
+    torch.cuda.synchronize()
+    for o in (opt, graphed, ranks[0][1], ranks[1][1]):
+        assert o.status() == 0 and o.ns_path() == L.LM_NS_F32_TC
+    assert sorted(set(own)) == [0, 1]
+    for i in range(len(shapes)):
+        np.testing.assert_array_equal(bits(replayed[i]), bits(eager[i]))
+        for p, _ in ranks:   # the update is a few percent of W, each within 2e-5
+            assert rel_fro(stored_values(p[i]), stored_values(eager[i])) <= 4e-6
 
 
 # ------------------------- beside other work -------------------------------
