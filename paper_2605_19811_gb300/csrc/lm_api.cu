@@ -563,8 +563,10 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
   }
   // The parts' workspace: at most kMaxPartBlocks blocks.  Where kcap asks for
   // more (15 layers of d = 4096, say), the shortest cap that fits bounds every
-  // tile, so that none is left whole.
-  const int64_t want = part;
+  // tile, so that none is left whole.  Without kcap the numbers of 128-column
+  // parts stay within 16 bits (only tiles above twice a worker's share are cut,
+  // a few hundred parts).
+  const int64_t want = part, most = kcap > 0 ? kMaxPartBlocks : kMaxPartBlocks / 2;
   std::vector<char> whole(ng, 0);
   int64_t planned;
   do {
@@ -572,12 +574,12 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
     planned = 0;
     for (int g = 0; g < ng; ++g) {
       const int64_t n = blocks[g] * std::min<int64_t>(64, (len[g] + part - 1) / part);
-      whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || (kcap <= 0 && planned + n > kMaxPartBlocks) ||
+      whole[g] = (len[g] <= keep && (kcap <= 0 || len[g] <= kcap)) || (kcap <= 0 && planned + n > most) ||
                  (kcap <= 0 && avg < 32 && len[g] - part < worth);
       if (!whole[g]) planned += n;
     }
     kcap += kcap > 0 ? 1 : 0;
-  } while (planned > kMaxPartBlocks && kcap <= longest);
+  } while (planned > most && kcap <= longest);
   std::vector<NsTile> out;
   nparts_total = 0;
   for (const NsTile& x0 : t) {

@@ -751,6 +751,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
   auto writes_global_w = [&](int ph, int it) {
     return fuse && ph == NS_APPLY && it == p.steps - 1 && !(p.it[it].mode & kIterFold);
   };
+  // Workspace tile of a split-K part.  Only the three-piece mode, whose cap cuts
+  // every long Gram tile, needs numbers past 16 bits (with them the bf16 epilogue
+  // spills more: ragged d = 300 set 231 us a Muon step against 228).
+  auto part_of = [](const NsTile& t) { return kP == 3 && !kPromo ? tc_part(t) : (int)t.slot - 1; };
   // epilogue reads the A (POLY) or X (APPLY) tile; an APPLY whose B has a
   // folded into its diagonal needs no X tile
   auto needs_aux = [&](int ph, int it) {
@@ -1179,7 +1183,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
           const int j = t.tn * kBN + c0;
           if (!inside(c0)) return;
           if (split)
-            split_chunk(x, p.split_ws + (size_t)tc_part(t) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN + c0,
+            split_chunk(x, p.split_ws + (size_t)part_of(t) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN + c0,
                         nscale, i < nrows, ncols - j);
           else
             piece_chunk<!kPromo>(x, phase, co, nscale, kacc, ap, aux, out, out_f32, plane, tile0 + c0, ld, i < nrows, j, ncols,
@@ -1234,7 +1238,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         }
       } else if (split) {
         // partial Gram product of a split tile: its own fp32 workspace tile
-        float* wrow = p.split_ws + (size_t)tc_part(t) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN;
+        float* wrow = p.split_ws + (size_t)part_of(t) * (BM * kBN) + (size_t)((int)rank * kHalf + row) * kBN;
 #pragma unroll 1
         for (int ch = half0 * (kBN / 64); ch < (half0 + nhalves) * (kBN / 64); ++ch) {
           uint32_t r[32];
@@ -1354,7 +1358,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
       // This warp's generic stores are ordered before its count (the reader's
       // proxy fence orders them before its TMA copies).
       if (lane == 0 && global_w) smem_counter_add(aux_left, 1u);
-      if (lane == 0 && split) red_release_gpu(p.parts_done + p.part_target[tc_part(t)], 1u);
+      if (lane == 0 && split) red_release_gpu(p.parts_done + p.part_target[part_of(t)], 1u);
       else if (lane == 0 && kP == 3) red_release_gpu(p.done + 3 * (size_t)(g.first_mat + t.mat) + phase, 1u);
     }
     if (kSplit)
