@@ -101,7 +101,11 @@ typedef struct {
  *                       of this state (or call) launched after it reads the
  *                       flag at entry and does nothing, so a step stops within
  *                       about one limit and writes no parameter after the
- *                       give-up, until lm_get_status clears the flag. */
+ *                       give-up, until lm_get_status clears the flag.  A
+ *                       Newton-Schulz launch of several phases also waits for
+ *                       other CTA pairs' tiles, up to the length of a phase
+ *                       (milliseconds on the largest sets): a limit below that
+ *                       gives up on steps that are well */
 
 /* Hyper-parameters: the Require line of Algorithm 1 plus the NS reading.
  * beta1, beta2 in [0, 1); eta_* >= 0; weight_decay >= 0;

@@ -281,12 +281,13 @@ constexpr int kSplitWorth = 48, kSplitWorthF32 = 6;
 // K blocks per CTA pair and iteration from which a batch runs one launch per
 // phase instead of one for the whole chain.  Such a batch works under the power
 // cap, where the chain's polls and its gapless run cost clocks as well as they
-// save gaps (2% of 2.1 ms an iteration): 720M-shaped set (6800 blocks), a Muon
-// and a Lion step sustained on three GPUs against the launches of the kernel
-// without the chain: one launch +1.1, -0.6 and -2%, a launch per phase 0 to
-// +0.5% (four GPUs); three-piece 4-layer d = 1280 set (4200) 7460 us in one
-// launch, 7370 per phase.  Below, one launch wins: 355M-shaped set (2600) 4.83 ms
-// per Muon step against 5.00, 124M-shaped 1515 us against 1672.
+// save gaps: a Muon and a Lion step of the 720M-shaped set (6800 blocks),
+// sustained, took -1.1, +0.6 and +2% of the time without the chain in one launch
+// on three GPUs, 0 to -0.5% in a launch per phase on four, where runs differ by
+// up to 2%; the three-piece 4-layer d = 1280 set (4200) 7460 us in one launch,
+// 7370 per phase.  Below, one launch wins: 355M-shaped set (2600) 4.83 ms per Muon
+// step against 5.00, 124M-shaped 1515 us against 1672.  No set between 2600 and
+// 4200 was measured; the line lies near the upper one.
 constexpr int kPhaseLaunchBlocks = 4096;
 // Largest msign workspace that stays in the stream-ordered pool until the
 // program's next synchronisation: 0.1% of the device, so that a caller's own
@@ -555,8 +556,9 @@ static void split_gram_tiles(const std::vector<NsGroup>& groups, int g0, int ng,
   // batch a whole embedding tile (786 blocks against a share of 305 on the 355M-
   // shaped set with a third of the matrices selected) would set the length of
   // the phase: no part longer than kMaskedGramPart (GRAM 298 -> 150 us per
-  // iteration there, the step 4658 -> 3957 us).  Without a mask it gains
-  // nothing (720M-shaped set: 1% slower for the summing).
+  // iteration there, the step 4658 -> 3957 us; no other set or share was
+  // measured).  Without a mask it gains nothing (720M-shaped set: 1% slower for
+  // the summing).
   if (masked && avg >= 32) {
     keep = std::min<int64_t>(keep, kMaskedGramPart);
     part = std::min<int64_t>(part, kMaskedGramPart);
@@ -1015,7 +1017,6 @@ static lm_status run_ns(const NsEngine& E, int steps, const NsCoeffs* coeffs, un
       c.pieces = E.pieces;
       c.promote = E.promote;
       c.bn = b.bn;
-      c.final_f32 = true;
       c.fuse = fuse;
       c.active = active;
       c.flags = flags;

@@ -201,8 +201,9 @@ struct NsCoeffs {
   float a, b, c, eps;
 };
 
-// Tensor-core path (bf16 operands, fp32 accumulation in TMEM): one
-// kTcBM x kTcBN output tile per CTA pair; s is padded to 128, l to kTcBN.
+// Tensor-core path (bf16 operands, fp32 accumulation in TMEM): one output tile
+// of kTcBM rows and kTcBN or 128 columns (tc_tile_cols; 128 always with three
+// pieces) per CTA pair; s is padded to 128, l to kTcBN.
 constexpr int kTcBM = 256, kTcBN = 256, kTcBK = 64;
 // Columns of a bf16 tile for a batch whose APPLY phase has `apply_tiles` tiles
 // of 256 x 256: 128 where that is at most one per CTA pair, 256 beyond.
@@ -293,7 +294,6 @@ struct NsChain {
   bool promote;                 // three pieces: main products summed in registers per K block (the full-fp32 mode)
   int bn;                       // columns of a tile: 256, or 128 (always with three pieces; not with a parameter
                                 // write whose iteration does not fold a)
-  bool final_f32;               // three pieces: the last APPLY writes fp32 X to NsGroup::Xf
   const FuseFinal* fuse;        // NULL, or the parameter write of the last APPLY (one piece)
   const unsigned char* active;  // NULL, or the mask the tile lists were compacted by
   unsigned* flags;
@@ -328,8 +328,8 @@ constexpr int kSimtBM = 128;   // s and l are padded to it
 int simt_pad(int x);
 int simt_blocks(int tile, int sms);   // resident blocks of the kernel for a tile
 // Tile of a phase with `tiles128` tiles of 128: 64 where those would leave more
-// than a fifth of the last round's blocks without work (or a single round
-// short), 128 otherwise.
+// than a fifth of the resident blocks, counted over all the rounds that the
+// tiles take, without work; 128 otherwise.
 int simt_tile(int64_t tiles128, int sms);
 constexpr int simt_slice(int tile) { return tile == 128 ? 16 : 32; }   // K slice (NsTile::kb0, kb1)
 // Split tiles (any phase): NsTile::slot = part + 1, nh = index << 8 | parts;

@@ -15,11 +15,11 @@
 // 64 (4 x 4 outputs, K slices of 32, four blocks per SM).  Slices are double-
 // buffered in shared memory: the global loads of slice k + 1 are in flight
 // while slice k is multiplied.
-// A phase that would leave more than a fifth of the resident 128-wide blocks
-// without work takes 64-wide ones, and where those leave blocks idle too, tiles
-// are cut along K: each part writes its partial tile, and the
-// block that finishes last adds the parts in order and writes the result, so
-// the sum does not depend on timing and nothing waits.
+// A phase that would leave more than a fifth of the resident 128-wide blocks,
+// over all its rounds, without work takes 64-wide ones, and where those leave
+// blocks idle too, tiles are cut along K: each part writes its partial tile, and
+// the block that finishes last adds the parts in order and writes the result,
+// so the sum does not depend on timing and nothing waits.
 // Same box, against 128-wide tiles only and a summing launch after each split
 // Gram: tiny fp32 set (256 x 256 to 256 x 1024, which now runs on the tensor
 // cores) 541 -> 314 us per Muon step, msign of 1024 x 1024 1497 -> 1026 us,

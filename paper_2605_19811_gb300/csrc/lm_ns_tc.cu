@@ -31,9 +31,10 @@
 // Measured on one box against one launch per phase with the epilogue warps
 // storing and waiting: 124M-shaped Muon step 1720 -> 1518 us, small sets
 // (2 layers, d = 128) 193 -> 109 us, one d = 768 layer from a graph 338 -> 231
-// us, three-piece 4-layer d = 1280 set 8030 -> 7460 us; in a launch per phase
-// that set 7300-7380 us, the 720M-shaped set (power-capped) 14.2-14.3 ms for a
-// Muon and a Lion step both ways.
+// us, three-piece 4-layer d = 1280 set 8030 -> 7460 us.  Large batches, which are
+// power-capped, take a launch per phase: that set 7300-7630 us over the GPUs
+// measured, the 720M-shaped set 14.2-14.7 ms for a Muon and a Lion step, no
+// different beyond noise from the kernel before the chain.
 //
 // CTA roles (384 threads, one CTA per SM; 12 warps, three per sub-partition):
 //   warp 0    TMA producer (one lane), smem ring (TcLayout); both CTAs' copies
@@ -451,7 +452,6 @@ struct ChainParams {
   unsigned* flags;
   FuseFinal fuse;            // fuse.mats != NULL: the last APPLY writes the parameters
   const unsigned char* active;
-  int final_f32;             // three-piece operands: the last APPLY writes fp32 X to NsGroup::Xf
   uint64_t wait_ns;
   ChainIter it[kMaxNsSteps];
 };
@@ -747,10 +747,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
   // memory after the tile (that phase then has a launch of its own, with
   // eight epilogue warps for the latency).
   const bool fuse = p.fuse.mats != nullptr;
-  // the parameter write that reads W from global memory (no TMA stores)
-  auto writes_global_w = [&](int ph, int it) {
-    return fuse && ph == NS_APPLY && it == p.steps - 1 && !(p.it[it].mode & kIterFold);
-  };
   // Workspace tile of a split-K part.  Only the three-piece mode, whose cap cuts
   // every long Gram tile, needs numbers past 16 bits (with them the bf16 epilogue
   // spills more: ragged d = 300 set 231 us a Muon step against 228).
@@ -1170,7 +1166,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
         const size_t plane = (size_t)g.count * msize;
         const __nv_bfloat16* aux = static_cast<const __nv_bfloat16*>(phase == NS_POLY ? g.A : g.X[cur]);
         __nv_bfloat16* out = static_cast<__nv_bfloat16*>(phase == NS_GRAM ? g.A : (phase == NS_POLY ? g.B : g.X[cur ^ 1]));
-        float* out_f32 = (phase == NS_APPLY && p.final_f32 && it == p.steps - 1) ? static_cast<float*>(g.Xf) : nullptr;
+        float* out_f32 = (phase == NS_APPLY && it == p.steps - 1) ? static_cast<float*>(g.Xf) : nullptr;
         // One 16-column chunk, columns [c0, c0 + 16) of the tile, next c0 + 16
         // of this warp's columns up to c1.  A chunk's aux values are loaded one
         // chunk ahead, the first before the accumulators are read.
@@ -1373,8 +1369,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kChainThreads, 1)
   }
 }
 
-// Split Gram tiles: bf16 A tile = the sum of the fp32 parts (already scaled),
-// added in part order.
+// Split Gram tiles of the wide kernel: bf16 A tile = the sum of the fp32 parts
+// (already scaled), added in part order.
 __global__ void __launch_bounds__(256) ns_split_finish_kernel(const NsSplitTarget* __restrict__ targets,
                                                               const float* __restrict__ ws, const unsigned* flags) {
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the Gram launch before it may be programmatic
@@ -1383,7 +1379,7 @@ __global__ void __launch_bounds__(256) ns_split_finish_kernel(const NsSplitTarge
   __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(T.a_tile);
   // four consecutive elements of a row per thread and trip (the tile's
   // column extent is a multiple of 128): 16-byte loads of every part, 8-byte
-  // stores per plane; each element's parts are still added in part order
+  // stores; each element's parts are still added in part order
   for (int e = (blockIdx.x * blockDim.x + threadIdx.x) * 4; e < BM * BN; e += gridDim.x * blockDim.x * 4) {
     const int r = e / BN, c = e % BN;
     if (r >= T.nr || c >= T.nc) continue;
@@ -1397,19 +1393,7 @@ __global__ void __launch_bounds__(256) ns_split_finish_kernel(const NsSplitTarge
       sum.z += v.z;
       sum.w += v.w;
     }
-    const size_t o = (size_t)r * T.ld + c;
-    if (T.plane == 0) {
-      *reinterpret_cast<uint2*>(dst + o) = make_uint2(pack_bf2(sum.x, sum.y), pack_bf2(sum.z, sum.w));
-    } else {   // three bf16 planes
-      float h[4], m[4], l[4];
-      split3(sum.x, h[0], m[0], l[0]);
-      split3(sum.y, h[1], m[1], l[1]);
-      split3(sum.z, h[2], m[2], l[2]);
-      split3(sum.w, h[3], m[3], l[3]);
-      *reinterpret_cast<uint2*>(dst + o) = make_uint2(pack_bf2(h[0], h[1]), pack_bf2(h[2], h[3]));
-      *reinterpret_cast<uint2*>(dst + T.plane + o) = make_uint2(pack_bf2(m[0], m[1]), pack_bf2(m[2], m[3]));
-      *reinterpret_cast<uint2*>(dst + 2 * T.plane + o) = make_uint2(pack_bf2(l[0], l[1]), pack_bf2(l[2], l[3]));
-    }
+    *reinterpret_cast<uint2*>(dst + (size_t)r * T.ld + c) = make_uint2(pack_bf2(sum.x, sum.y), pack_bf2(sum.z, sum.w));
   }
 }
 
@@ -1688,7 +1672,6 @@ static cudaError_t launch_chain_part(const NsChain& c, int q0, int q1, ChainPart
   prm.steps = c.steps;
   prm.flags = c.flags;
   prm.active = c.active;
-  prm.final_f32 = c.pieces == 3 && c.final_f32 ? 1 : 0;
   prm.wait_ns = c.wait_ns;
   uint32_t npoly = 0;
   for (int it = 0; it < c.steps; ++it) {

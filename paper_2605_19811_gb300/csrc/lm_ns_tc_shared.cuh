@@ -1,6 +1,7 @@
 // Definitions shared by the two tensor-core Newton-Schulz kernels:
-//   lm_ns_tc.cu   one 256 x 256 output tile per CTA pair, two accumulators
-//                 in TMEM (bf16 operands, or fp32 as three bf16 pieces);
+//   lm_ns_tc.cu   one output tile of 256 x 256 or 256 x 128 per CTA pair (bf16
+//                 operands; 256 x 128 for fp32 as three bf16 pieces), two
+//                 tiles' accumulators in TMEM;
 //   lm_ns_wide.cu tiles of one or two 256-column halves per CTA pair (bf16),
 //                 which reuse one staged A box for both halves.
 // Both run the NS phases of Section 2's iteration (GRAM A = X X^T, POLY
