@@ -292,8 +292,8 @@ constexpr int kPhaseLaunchBlocks = 4096;
 // Largest msign workspace that stays in the stream-ordered pool until the
 // program's next synchronisation: 0.1% of the device, so that a caller's own
 // allocation after the call does not miss it.  Past it the memory's return and
-// renewal cost 0.5 ms (4096 x 4096 bf16, 1.0 ms) to 3.5 ms a call (50304 x 2048
-// fp32, 14.9 ms).
+// renewal cost 1.5 ms a call (50304 x 768 fp32, 3.5 ms without) to 3.6 ms (50304 x
+// 2048 fp32, 14.9 ms).
 constexpr size_t kMsignKeepBytes = (size_t)256 << 20;
 constexpr uint64_t kRingWaitNs = 2000000000ull;   // the power-iteration ring's waits: 2 s unless set shorter
 
